@@ -48,7 +48,7 @@ def source_hash() -> str:
     return h.hexdigest()[:16]
 
 
-KERNEL_SOURCES = ("fft_codelets.cuh", "fft_plan.h", "hfx_kernels.cuh", "hfx_ct.cuh")
+KERNEL_SOURCES = ("fft_codelets.cuh", "fft_plan.h", "hfx_kernels.cuh", "hfx_ct.cuh", "hfx_ct_plane.cuh")
 
 
 def kernel_hash() -> str:

@@ -31,6 +31,48 @@ template <typename C> __device__ __forceinline__ C cmul(C a, C b) {
 template <typename C> __device__ __forceinline__ C cmulc(C a, C b) {
   return mk<C>(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
 }
+// FP32 pairs in one instruction (add.f32x2 and so on round each half like the scalar instruction): the
+// FMA pipe takes them at the same rate per element, but they need half the issue slots, which bound the
+// plane passes
+__device__ __forceinline__ unsigned long long pack2(float2 a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+  return r;
+}
+template <> __device__ __forceinline__ float2 cadd<float2>(float2 a, float2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+  return unpack2(r);
+}
+template <> __device__ __forceinline__ float2 csub<float2>(float2 a, float2 b) {
+  unsigned long long r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+  return unpack2(r);
+}
+// a + s i b and a + c b for a real constant c, with multiply-adds where they are products
+template <int S, typename C> __device__ __forceinline__ C cadd_si(C a, C b) {
+  if constexpr (S > 0) return mk<C>(a.x - b.y, a.y + b.x);
+  else return mk<C>(a.x + b.y, a.y - b.x);
+}
+template <int S, typename C> __device__ __forceinline__ C cfma_si(C a, C b, decltype(C::x) c) {
+  if constexpr (S > 0) return mk<C>(a.x - c * b.y, a.y + c * b.x);
+  else return mk<C>(a.x + c * b.y, a.y - c * b.x);
+}
+template <typename C> __device__ __forceinline__ C cfma(C a, C b, decltype(C::x) c) {
+  return mk<C>(a.x + c * b.x, a.y + c * b.y);
+}
+#ifdef PACKFMA
+template <> __device__ __forceinline__ float2 cfma<float2>(float2 a, float2 b, float c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack2(b)), "l"(pack2(make_float2(c, c))), "l"(pack2(a)));
+  return unpack2(r);
+}
+#endif
 // s * i * a, s = +-1 (compile time)
 template <int S, typename C> __device__ __forceinline__ C mul_si(C a) {
   if constexpr (S > 0) return mk<C>(-a.y, a.x);
@@ -132,22 +174,21 @@ template <int DIR, typename C> struct Dft<3, DIR, C> {
     constexpr T s3 = T(0.86602540378443864676372317075293618347);  // sin(2 pi / 3)
     C t1 = cadd(x[1], x[2]);
     C d = csub(x[1], x[2]);
-    C a = mk<C>(x[0].x - T(0.5) * t1.x, x[0].y - T(0.5) * t1.y);
-    C b = mul_si<DIR>(cscale(d, s3));  // DIR i s3 (x1 - x2)
+    C a = cfma(x[0], t1, T(-0.5));
     x[0] = cadd(x[0], t1);
-    x[1] = cadd(a, b);
-    x[2] = csub(a, b);
+    x[1] = cfma_si<DIR>(a, d, s3);  // a +- DIR i s3 (x1 - x2)
+    x[2] = cfma_si<-DIR>(a, d, s3);
   }
 };
 
 template <int DIR, typename C> struct Dft<4, DIR, C> {
   static __device__ __forceinline__ void run(C (&x)[4]) {
     C s02 = cadd(x[0], x[2]), d02 = csub(x[0], x[2]);
-    C s13 = cadd(x[1], x[3]), d13 = mul_si<DIR>(csub(x[1], x[3]));
+    C s13 = cadd(x[1], x[3]), d13 = csub(x[1], x[3]);
     x[0] = cadd(s02, s13);
     x[2] = csub(s02, s13);
-    x[1] = cadd(d02, d13);
-    x[3] = csub(d02, d13);
+    x[1] = cadd_si<DIR>(d02, d13);
+    x[3] = cadd_si<-DIR>(d02, d13);
   }
 };
 
@@ -160,15 +201,13 @@ template <int DIR, typename C> struct Dft<5, DIR, C> {
     constexpr T s2 = T(0.58778525229247312916870595463907276860);   // sin(4 pi/5)
     C a1 = cadd(x[1], x[4]), b1 = csub(x[1], x[4]);
     C a2 = cadd(x[2], x[3]), b2 = csub(x[2], x[3]);
-    C r1 = mk<C>(x[0].x + c1 * a1.x + c2 * a2.x, x[0].y + c1 * a1.y + c2 * a2.y);
-    C r2 = mk<C>(x[0].x + c2 * a1.x + c1 * a2.x, x[0].y + c2 * a1.y + c1 * a2.y);
-    C i1 = mul_si<DIR>(mk<C>(s1 * b1.x + s2 * b2.x, s1 * b1.y + s2 * b2.y));
-    C i2 = mul_si<DIR>(mk<C>(s2 * b1.x - s1 * b2.x, s2 * b1.y - s1 * b2.y));
+    C r1 = cfma(cfma(x[0], a1, c1), a2, c2);
+    C r2 = cfma(cfma(x[0], a1, c2), a2, c1);
     x[0] = cadd(x[0], cadd(a1, a2));
-    x[1] = cadd(r1, i1);
-    x[4] = csub(r1, i1);
-    x[2] = cadd(r2, i2);
-    x[3] = csub(r2, i2);
+    x[1] = cfma_si<DIR>(cfma_si<DIR>(r1, b1, s1), b2, s2);
+    x[4] = cfma_si<-DIR>(cfma_si<-DIR>(r1, b1, s1), b2, s2);
+    x[2] = cfma_si<DIR>(cfma_si<DIR>(r2, b1, s2), b2, -s1);
+    x[3] = cfma_si<-DIR>(cfma_si<-DIR>(r2, b1, s2), b2, -s1);
   }
 };
 
@@ -199,6 +238,33 @@ __device__ __forceinline__ void dft_composite(C (&x)[P * Q]) {
   }
 }
 
+// R = P * Q with P and Q coprime (Good-Thomas): input j = Q j1 + P j2 mod R, output k with
+// k = k1 mod P and k = k2 mod Q; no twiddles between the two factors.
+template <int P, int Q, int DIR, typename C>
+__device__ __forceinline__ void dft_coprime(C (&x)[P * Q]) {
+  constexpr int R = P * Q;
+  C y[R];
+  static_for<0, Q>([&](auto J2) {
+    constexpr int j2 = decltype(J2)::value;
+    C t[P];
+    static_for<0, P>([&](auto J1) { t[decltype(J1)::value] = x[(Q * decltype(J1)::value + P * j2) % R]; });
+    Dft<P, DIR, C>::run(t);
+#pragma unroll
+    for (int k1 = 0; k1 < P; ++k1) y[k1 * Q + j2] = t[k1];
+  });
+  C z[R];
+#pragma unroll
+  for (int k1 = 0; k1 < P; ++k1) {
+    C t[Q];
+#pragma unroll
+    for (int j2 = 0; j2 < Q; ++j2) t[j2] = y[k1 * Q + j2];
+    Dft<Q, DIR, C>::run(t);
+#pragma unroll
+    for (int k2 = 0; k2 < Q; ++k2) z[k1 * Q + k2] = t[k2];
+  }
+  static_for<0, R>([&](auto K) { x[decltype(K)::value] = z[(decltype(K)::value % P) * Q + decltype(K)::value % Q]; });
+}
+
 template <int DIR, typename C> struct Dft<6, DIR, C> {
   static __device__ __forceinline__ void run(C (&x)[6]) { dft_composite<2, 3, DIR>(x); }
 };
@@ -216,6 +282,18 @@ template <int DIR, typename C> struct Dft<12, DIR, C> {
 };
 template <int DIR, typename C> struct Dft<16, DIR, C> {
   static __device__ __forceinline__ void run(C (&x)[16]) { dft_composite<4, 4, DIR>(x); }
+};
+template <int DIR, typename C> struct Dft<18, DIR, C> {
+  static __device__ __forceinline__ void run(C (&x)[18]) { dft_coprime<2, 9, DIR>(x); }
+};
+template <int DIR, typename C> struct Dft<20, DIR, C> {
+  static __device__ __forceinline__ void run(C (&x)[20]) { dft_coprime<4, 5, DIR>(x); }
+};
+template <int DIR, typename C> struct Dft<24, DIR, C> {
+  static __device__ __forceinline__ void run(C (&x)[24]) { dft_coprime<8, 3, DIR>(x); }
+};
+template <int DIR, typename C> struct Dft<32, DIR, C> {
+  static __device__ __forceinline__ void run(C (&x)[32]) { dft_composite<4, 8, DIR>(x); }
 };
 
 }  // namespace hfx

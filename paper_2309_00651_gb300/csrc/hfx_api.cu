@@ -137,14 +137,14 @@ static bool encode_f32_4d(CUtensorMap* m, const void* base, const cuuint64_t dim
 
 // the maps of the TMA dense accumulate pass (tiles it reads; V also the tensor its reduce-adds
 // write) for a cubic grid of edge n: a transform buffer of
-// `cap` couples, W[couple][x][y][z] complex FP32, as (z reals, couple, y, x) with boxes of 8
+// `cap` couples, complex FP32 with element strides wx and wy of x and y, as (z reals, couple, y, x) with boxes of 8
 // complex x `cpi` couples x n rows; the FP32 orbitals orb[orbital][x][y][z] and the FP32
 // accumulator V (same layout) as (z, y, orbital, x) with boxes of 8 x n x 8
-static bool encode_dense_maps(CUtensorMap* tmW, const void* W, long long cap, int cpi, CUtensorMap* tmOrb,
+static bool encode_dense_maps(CUtensorMap* tmW, const void* W, long long cap, int cpi, int wx, int wy, CUtensorMap* tmOrb,
                               const void* orb, CUtensorMap* tmV, const void* V, int n_orb, int n) {
   const cuuint64_t nn = (cuuint64_t)n, N3 = nn * nn * nn;
   const cuuint64_t dw[4] = {2 * nn, (cuuint64_t)cap, nn, nn};
-  const cuuint64_t sw[3] = {N3 * 8, nn * 8, nn * nn * 8};
+  const cuuint64_t sw[3] = {N3 * 8, (cuuint64_t)wy * 8, (cuuint64_t)wx * 8};
   const cuuint32_t bw[4] = {16, (cuuint32_t)cpi, (cuuint32_t)n, 1};
   const cuuint64_t dorb[4] = {nn, nn, (cuuint64_t)n_orb, nn};
   const cuuint64_t sorb[3] = {nn * 4, N3 * 4, nn * nn * 4};
@@ -188,7 +188,8 @@ struct hfx_ctx {
   int rb = 0;
   // compile-time-geometry passes (FP32, cubic grid with an instantiated edge), else NULL
   const CtFns* ct = nullptr;
-  void* d_twct = nullptr;        // per-stage twiddle tables of the edge
+  void* d_twct = nullptr;        // per-stage twiddle tables of the edge (accumulate passes)
+  void* d_twplane = nullptr;     // twiddles of the forward and x passes
   int blocks_fwd_ct = 1, blocks_x_ct = 1;
   // the compile-time dense accumulate pass moves its tiles by TMA (HFX_DENSE_TMA=0: per-thread
   // asynchronous copies)
@@ -285,7 +286,6 @@ static size_t smem_dense(const hfx_ctx* c) {
   return (size_t)(kDenseRing * c->grid[1] * (c->bsize / 2) * zc + c->grid[1]) * cplx_size(c) +
          (size_t)2 * c->bsize * c->grid[1] * zc * real_size(c);
 }
-static size_t smem_plane_ct(int n) { return (size_t)(n * (n + 1) + stage_plan(n).twtotal) * sizeof(float2); }
 static size_t smem_dense_ct(int n, int b) {
   const int zc = 8, ln = dense_rows_ct(n) * (b / 2) * zc, pts = n * zc;
   return (size_t)(kDenseRingCt * n * ln + stage_plan(n).twtotal) * sizeof(float2) + (size_t)2 * b * pts * sizeof(float);
@@ -313,6 +313,39 @@ static std::vector<double> stage_twiddles(int n) {
       }
   }
   return tw;
+}
+
+// the edges whose forward and x passes are the plane passes (hfx_ct_plane.cuh): z and x split (n / 4) x 4
+static bool plane_edge(int n) { return n % 8 == 0; }
+
+// twiddles of the forward and x passes of edge n: w_n^{e k}, e < 4, k < n / 4 at ((k / 2) 4 + e) 2 + k % 2,
+// then y's first stage [j][k]; the stage tables where the passes run one stage at a time
+static std::vector<double> plane_twiddles(int n) {
+  if (!plane_edge(n)) return stage_twiddles(n);
+  const StagePlan y = stage_plan(n);
+  const int R = n / 4;
+  std::vector<double> tw(2 * (size_t)(4 * R + y.r[0] * y.m[0]));
+  for (int e = 0; e < 4; ++e)
+    for (int k = 0; k < R; ++k) {
+      const cs_pair w = cossin_2pi_frac((long long)e * k, n);
+      const size_t idx = (size_t)((k / 2) * 4 + e) * 2 + k % 2;
+      tw[2 * idx] = w.c;
+      tw[2 * idx + 1] = -w.s;
+    }
+  const std::vector<double> ty = stage_twiddles(n);
+  std::copy_n(ty.begin(), 2 * (size_t)(y.r[0] * y.m[0]), tw.begin() + 2 * (size_t)(4 * R));
+  return tw;
+}
+
+// the split of z and x of a plane edge
+static void set_plane_plan(DimPlan& d) {
+  d.ns = 2;
+  d.r[0] = d.n / 4;
+  d.m[0] = 4;
+  d.r[1] = 4;
+  d.m[1] = 1;
+  for (int s = 2; s < kMaxStages; ++s) { d.r[s] = 1; d.m[s] = 1; }
+  for (int s = 0; s < kMaxStages; ++s) d.mdiv[s] = FastDiv::make((uint32_t)d.m[s]);
 }
 
 // pencil kernels: rows blocks of rb rows (padded stride n3 + 1) and single z-chunk columns
@@ -381,6 +414,8 @@ static void free_ctx_tables(hfx_ctx* c) {
   c->side = nullptr;
   dev_free(c->d_twct);
   c->d_twct = nullptr;
+  dev_free(c->d_twplane);
+  c->d_twplane = nullptr;
   dev_free(c->d_batch);
   c->d_batch = nullptr;
   dev_free(c->d_dftb);
@@ -554,6 +589,8 @@ extern "C" hfx_status hfx_create(const hfx_box* box, const int32_t grid[3], doub
   }
   c->N = (long long)grid[0] * grid[1] * grid[2];
   c->geo.n1 = grid[0]; c->geo.n2 = grid[1]; c->geo.n3 = grid[2]; c->geo.N = c->N;
+  c->geo.wx = grid[1] * grid[2];
+  c->geo.wy = grid[2];
   c->geo.S = grid[2] + 1;  // odd row stride: column accesses of consecutive lines hit distinct banks
   std::memcpy(c->lat, box->lattice, sizeof(c->lat));
   const double (*A)[3] = c->lat;
@@ -606,6 +643,22 @@ extern "C" hfx_status hfx_create(const hfx_box* box, const int32_t grid[3], doub
   }
   c->blocks_fwd = std::max(1, c->blocks_fwd);
   c->blocks_x = std::max(1, c->blocks_x);
+  // compile-time-geometry passes for FP32 cubic grids with an instantiated edge; their split of z and x,
+  // and where they keep x and y in the transforms, also hold for the tables and the generic pass
+  const char* no_ct = std::getenv("HFX_NO_CT");
+  const int n = grid[0];
+  if (prec == HFX_PREC_FP32 && !c->pencil && grid[0] == grid[1] && grid[1] == grid[2] && !(no_ct && atoi(no_ct) != 0)) {
+    const CtFns* f = ct_fns(n);
+    if (f && std::max({f->smem_plane, smem_dense_tma_ct(n), smem_diag_ct(n, 8) + 128}) + 512 <= (size_t)c->max_smem) {
+      c->ct = f;
+      if (plane_edge(n)) {
+        set_plane_plan(c->geo.d[0]);
+        set_plane_plan(c->geo.d[2]);
+        c->geo.wx = n;
+        c->geo.wy = n * n;
+      }
+    }
+  }
   hfx_status st = build_tables(c.get());
   if (st != HFX_OK) { free_ctx_tables(c.get()); return st; }
   {
@@ -617,33 +670,31 @@ extern "C" hfx_status hfx_create(const hfx_box* box, const int32_t grid[3], doub
       return fail(HFX_ERR_CUDA, "stream/event creation failed: %s", cudaGetErrorString(es));
     }
   }
-  // compile-time-geometry passes for FP32 cubic grids with an instantiated edge
-  const char* no_ct = std::getenv("HFX_NO_CT");
-  if (prec == HFX_PREC_FP32 && !c->pencil && grid[0] == grid[1] && grid[1] == grid[2] && !(no_ct && atoi(no_ct) != 0)) {
-    const CtFns* f = ct_fns(grid[0]);
-    const int n = grid[0];
-    if (f && std::max({smem_plane_ct(n), smem_dense_tma_ct(n), smem_diag_ct(n, 8) + 128}) + 512 <= (size_t)c->max_smem) {
-      e = f->prepare(c->max_smem - 512, smem_plane_ct(n), &c->blocks_fwd_ct, &c->blocks_x_ct);
-      if (e != cudaSuccess) { free_ctx_tables(c.get()); return fail(HFX_ERR_CUDA, "kernel setup: %s", cudaGetErrorString(e)); }
-      auto tw = to_real_vec<float>(stage_twiddles(n));
-      st = upload(&c->d_twct, tw.data(), tw.size() * sizeof(float));
-      if (st != HFX_OK) { free_ctx_tables(c.get()); return st; }
-      c->blocks_fwd_ct = std::max(1, c->blocks_fwd_ct);
-      c->blocks_x_ct = std::max(1, c->blocks_x_ct);
-      c->ct = f;
-      // TMA needs the driver's tensor-map encoder; without it the dense pass copies per thread
-      if (!encode_tiled()) c->dense_tma = false;
+  if (c->ct) {
+    e = c->ct->prepare(c->max_smem - 512, &c->blocks_fwd_ct, &c->blocks_x_ct);
+    if (e != cudaSuccess) { free_ctx_tables(c.get()); return fail(HFX_ERR_CUDA, "kernel setup: %s", cudaGetErrorString(e)); }
+    auto tw = to_real_vec<float>(stage_twiddles(n));
+    st = upload(&c->d_twct, tw.data(), tw.size() * sizeof(float));
+    if (st == HFX_OK) {
+      tw = to_real_vec<float>(plane_twiddles(n));
+      st = upload(&c->d_twplane, tw.data(), tw.size() * sizeof(float));
     }
+    if (st != HFX_OK) { free_ctx_tables(c.get()); return st; }
+    c->blocks_fwd_ct = std::max(1, c->blocks_fwd_ct);
+    c->blocks_x_ct = std::max(1, c->blocks_x_ct);
+    // TMA needs the driver's tensor-map encoder; without it the dense pass copies per thread
+    if (!encode_tiled()) c->dense_tma = false;
   }
   if (mixed_tc) {
-    const int n = grid[0];
     if (!c->ct || !dft::tc_edge(n))
       return fail(HFX_ERR_UNSUPPORTED_GRID,
                   "HFX_PREC_MIXED_TC needs a cubic grid of edge 32, 48, 64 or 96 (got %d x %d x %d)", (int)grid[0],
                   (int)grid[1], (int)grid[2]);
     e = dft::tc_prepare(n, &c->blocks_fwd_tc);
     if (e != cudaSuccess) { free_ctx_tables(c.get()); return fail(HFX_ERR_CUDA, "kernel setup: %s", cudaGetErrorString(e)); }
-    const std::vector<uint32_t> tb = dft_tc_table(c->geo.d[2]);
+    std::vector<uint32_t> tb = dft_tc_table(c->geo.d[2]);  // z, then y
+    const std::vector<uint32_t> tby = dft_tc_table(c->geo.d[1]);
+    tb.insert(tb.end(), tby.begin(), tby.end());
     st = upload(&c->d_dftb, tb.data(), tb.size() * sizeof(uint32_t));
     if (st != HFX_OK) { free_ctx_tables(c.get()); return st; }
     c->blocks_fwd_tc = std::max(1, c->blocks_fwd_tc);
@@ -979,8 +1030,8 @@ static hfx_status run_passes(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
   if (std::is_same<T, float>::value && c->ct && S.b == 8 && c->dense_tma && !energy_only && g.n1 % 4 == 0) {
     const int cpi = dense_rows_ct(g.n1) * (S.b / 2);
     dense_tma =
-        encode_dense_maps(&tmW[0], Wbuf[0], S.max_batch_couples, cpi, &tmOrb, orb, &tmV, vacc, n_orb, g.n1) &&
-        encode_dense_maps(&tmW[1], Wbuf[1], S.max_batch_couples, cpi, &tmOrb, orb, &tmV, vacc, n_orb, g.n1);
+        encode_dense_maps(&tmW[0], Wbuf[0], S.max_batch_couples, cpi, g.wx, g.wy, &tmOrb, orb, &tmV, vacc, n_orb, g.n1) &&
+        encode_dense_maps(&tmW[1], Wbuf[1], S.max_batch_couples, cpi, g.wx, g.wy, &tmOrb, orb, &tmV, vacc, n_orb, g.n1);
     // the buffers are 16-byte aligned and the edges multiples of 4, so the driver has no reason to refuse
     if (!dense_tma) return fail(HFX_ERR_CUDA, "cuTensorMapEncodeTiled refused the dense pass's tensor maps");
   }
@@ -1024,8 +1075,8 @@ static hfx_status run_passes(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
                        (const unsigned char*)c->d_dftb, c->d_err);
       } else if (ct) {
         const int gct = (int)std::min<long long>(items1, (long long)c->sm_count * c->blocks_fwd_ct * c->ct_waves);
-        ct->fwd_yz(std::max(gct, 1), smem_plane_ct(g.n1), fs, (const float*)orb, g.N, couples, c0, c1, (float2*)W,
-                   (const float2*)c->d_twct, c->prefetch ? 1 : 0);
+        ct->fwd_yz(std::max(gct, 1), fs, (const float*)orb, g.N, couples, c0, c1, (float2*)W,
+                   (const float2*)c->d_twplane, c->prefetch ? 1 : 0);
       } else {
         Passes<T>::fwd_yz(g, std::max(grid1, 1), smem_fwd(c), fs, orb, couples, c0, c1, W, (const C*)c->d_tw[1],
                           (const C*)c->d_tw[2]);
@@ -1034,8 +1085,8 @@ static hfx_status run_passes(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
       e0 = mark(fs);
       if (ct) {
         const int gct = (int)std::min<long long>(items2, (long long)c->sm_count * c->blocks_x_ct * c->ct_waves);
-        ct->x_coulomb(std::max(gct, 1), smem_plane_ct(g.n1), fs, couples, c0, c1, (float2*)W, (const float*)c->d_vtab,
-                      (const float2*)c->d_twct, epart, energy_only ? 1 : 0, c->prefetch ? 1 : 0);
+        ct->x_coulomb(std::max(gct, 1), fs, couples, c0, c1, (float2*)W, (const float*)c->d_vtab,
+                      (const float2*)c->d_twplane, epart, energy_only ? 1 : 0, c->prefetch ? 1 : 0);
       } else {
         Passes<T>::x_coulomb(g, std::max(grid2, 1), smem_x(c), fs, couples, c0, c1, W, (const T*)c->d_vtab,
                              (const C*)c->d_tw[0], (const C*)c->d_tw[2], epart, energy_only ? 1 : 0);
@@ -1300,11 +1351,8 @@ static hfx_status batched_persistent(hfx_ctx* const* ctxs, const hfx_apply_args*
     P.tw3 = (const cx<T>*)c->d_tw[2];
     P.slot_couple_base = S->d_slot_couple_base;
     P.slot_blocks = S->d_slot_blocks;
-    P.twct = (const cx<T>*)c->d_twct;
-    P.ct_n = (std::is_same<T, float>::value && c->ct && (c->grid[0] == 48 || c->grid[0] == 64 || c->grid[0] == 72 ||
-                                                        c->grid[0] == 80 || c->grid[0] == 90 || c->grid[0] == 96))
-                 ? c->grid[0]
-                 : 0;
+    P.twct = (const cx<T>*)c->d_twplane;
+    P.ct_n = std::is_same<T, float>::value && c->ct ? c->grid[0] : 0;
     P.err = c->d_err;
     P.vscale = -c->alpha / (double)c->N;
     P.escale = -0.5 * c->alpha * c->omega / ((double)c->N * (double)c->N);
@@ -1342,7 +1390,7 @@ static hfx_status batched_persistent(hfx_ctx* const* ctxs, const hfx_apply_args*
     if (std::is_same<T, float>::value && !eo) add(kTaskWiden, (P.n_v + kWidenPerItem - 1) / kWidenPerItem, 0, 0, 0);
     add(kTaskEnergy, 1, 0, 0, 0);
     chains.push_back(ch);
-    smem = std::max({smem, smem_fwd(c), smem_x(c)});
+    smem = std::max(smem, P.ct_n ? c->ct->smem_plane : std::max(smem_fwd(c), smem_x(c)));
   }
   if (probs.empty()) return HFX_OK;
   // the accumulate tiles take at most the planes' footprint (largest couple group and orbital

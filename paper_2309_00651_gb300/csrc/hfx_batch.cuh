@@ -22,12 +22,14 @@
 #include <type_traits>
 
 #include "hfx_ct.cuh"
+#include "hfx_ct_plane.cuh"
 #include "hfx_kernels.cuh"
 
 namespace hfx {
 
 enum BatchKind : int { kTaskFwd = 0, kTaskX = 1, kTaskAcc = 2, kTaskEnergy = 3, kTaskWiden = 4 };
 
+constexpr int kThreadsBatch = 256;
 constexpr int kWidenPerItem = 4096;  // elements of V_x phi per widening item
 
 template <typename T>
@@ -47,7 +49,7 @@ struct BatchProblem {
   const cx<T>* tw3;
   const int* slot_couple_base;
   const int2* slot_blocks;
-  const cx<T>* twct;            // per-stage twiddles of the compile-time passes (ct_n > 0)
+  const cx<T>* twct;            // twiddles of the compile-time forward and x passes (ct_n > 0)
   int* err;                     // the problem's context error word
   double vscale, escale;
   int n_orb, bsize, grp, phi_smem, cap_max, total_couples, accumulate, energy_only;
@@ -62,16 +64,33 @@ __device__ __forceinline__ bool ct_item_n(const BatchProblem<T>& P, int kind, in
                                           unsigned char* smem_raw, float (*redf)[32], int par, bool tw_ok) {
   if constexpr (std::is_same<T, float>::value) {
     if (P.ct_n != N) return false;
-    constexpr StagePlan SP = ct::Plan<N>::p;
-    float2* buf = reinterpret_cast<float2*>(smem_raw);
-    float2* tw = buf + N * (N + 1);
-    if (!tw_ok)
-      for (int i = threadIdx.x; i < SP.twtotal; i += blockDim.x) tw[i] = P.twct[i];
-    if (kind == kTaskFwd)
-      ct::fwd_yz_ct_item<float, N>(P.orb, P.g.N, P.couples, a0, P.W, buf, tw, (int)local);
-    else
-      ct::x_coulomb_ct_item<float, N>(P.couples, a0, P.W, P.vtab, P.epart, P.energy_only, buf, tw, redf, par,
-                                      (int)local);
+    if constexpr (N % 8 == 0) {
+      using G = ct::PlaneGeo<N>;
+      float2* tw = reinterpret_cast<float2*>(smem_raw);
+      float2* buf = tw + G::TW + G::TWY;
+      if (!tw_ok) {
+        for (int i = threadIdx.x; i < G::TW + G::TWY; i += blockDim.x) tw[i] = P.twct[i];
+        __syncthreads();
+      }
+      const int cl = (int)local / N, pl = (int)local - cl * N;
+      const int4 cp = P.couples[a0 + cl];
+      if (couple_empty(cp)) return true;
+      if (kind == kTaskFwd)
+        ct::fwd_plane_item<N, kThreadsBatch, 2>(P.orb, P.g.N, cp, P.W, buf, tw, cl, pl);
+      else
+        ct::x_plane_item<N, kThreadsBatch>(a0, P.W, P.vtab, P.epart, P.energy_only, buf, tw, redf, par, cl, pl);
+    } else {
+      constexpr StagePlan SP = ct::Plan<N>::p;
+      float2* buf = reinterpret_cast<float2*>(smem_raw);
+      float2* tw = buf + N * (N + 1);
+      if (!tw_ok)
+        for (int i = threadIdx.x; i < SP.twtotal; i += blockDim.x) tw[i] = P.twct[i];
+      if (kind == kTaskFwd)
+        ct::fwd_yz_ct_item<float, N>(P.orb, P.g.N, P.couples, a0, P.W, buf, tw, (int)local);
+      else
+        ct::x_coulomb_ct_item<float, N>(P.couples, a0, P.W, P.vtab, P.epart, P.energy_only, buf, tw, redf, par,
+                                        (int)local);
+    }
     return true;
   } else {
     return false;
@@ -81,12 +100,14 @@ __device__ __forceinline__ bool ct_item_n(const BatchProblem<T>& P, int kind, in
 template <typename T>
 __device__ __forceinline__ bool ct_item(const BatchProblem<T>& P, int kind, int a0, long long local,
                                         unsigned char* smem_raw, float (*redf)[32], int par, bool tw_ok) {
-  return ct_item_n<T, 48>(P, kind, a0, local, smem_raw, redf, par, tw_ok) ||
+  return ct_item_n<T, 32>(P, kind, a0, local, smem_raw, redf, par, tw_ok) ||
+         ct_item_n<T, 48>(P, kind, a0, local, smem_raw, redf, par, tw_ok) ||
          ct_item_n<T, 64>(P, kind, a0, local, smem_raw, redf, par, tw_ok) ||
          ct_item_n<T, 72>(P, kind, a0, local, smem_raw, redf, par, tw_ok) ||
          ct_item_n<T, 80>(P, kind, a0, local, smem_raw, redf, par, tw_ok) ||
          ct_item_n<T, 90>(P, kind, a0, local, smem_raw, redf, par, tw_ok) ||
-         ct_item_n<T, 96>(P, kind, a0, local, smem_raw, redf, par, tw_ok);
+         ct_item_n<T, 96>(P, kind, a0, local, smem_raw, redf, par, tw_ok) ||
+         ct_item_n<T, 128>(P, kind, a0, local, smem_raw, redf, par, tw_ok);
 }
 
 struct BatchTask {
@@ -114,7 +135,6 @@ __device__ __forceinline__ int ld_acquire_gpu(const int* p) {
   return v;
 }
 
-constexpr int kThreadsBatch = 256;
 // resident blocks per SM the persistent kernel is built for (registers: FP64 items need more)
 template <typename T> struct BatchMinBlocks { static constexpr int value = sizeof(T) == 4 ? 3 : 1; };
 

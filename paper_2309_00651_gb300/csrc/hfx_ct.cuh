@@ -14,6 +14,13 @@ namespace ct {
 
 template <int N> struct Plan { static constexpr StagePlan p = stage_plan(N); };
 
+// element strides of x and y in a couple's transform W: [y][x][z] where the plane passes of
+// hfx_ct_plane.cuh run (edges that are a multiple of 8), else [x][y][z]
+template <int N> struct WStride {
+  static constexpr int x = N % 8 == 0 ? N : N * N;
+  static constexpr int y = N % 8 == 0 ? N * N : N;
+};
+
 // one in-place stage over LINES lines (element e of line l at buf[l*LS + e*ES])
 template <int R, int M, bool INV, int LINES, int LS, int ES, int N, int NT, typename C>
 __device__ __forceinline__ void stage(C* __restrict__ buf, const C* __restrict__ twt) {
@@ -493,7 +500,7 @@ k_y_acc_dense_ct(const T* __restrict__ orb, long long Ntot, const int4* __restri
       const int ut = rest % (RPI * HB), y = rest / (RPI * HB);  // ut = u * HB + t
       const int cr = k * RPI * HB + ut;                          // couple within the block pair
       const bool ok_c = ((live >> cr) & 1u) && v * PER < zcn;
-      const C* src = W + ((long long)(cs + cr - c0) * N + x) * PLANE + (long long)y * N + z0 + v * PER;
+      const C* src = W + (long long)(cs + cr - c0) * N * PLANE + x * WStride<N>::x + y * WStride<N>::y + z0 + v * PER;
       cp_async16(dstb + y * LN + ut * ZC + v * PER, ok_c ? (const void*)src : (const void*)W, ok_c ? 16 : 0);
     }
     cp_async_commit();

@@ -2,6 +2,7 @@
 // edge, so the sizes compile in parallel).
 #include "hfx_ct.cuh"
 #include "hfx_ct_diag.cuh"
+#include "hfx_ct_plane.cuh"
 #include "hfx_internal.h"
 
 namespace hfx {
@@ -9,34 +10,46 @@ namespace {
 
 constexpr int kN = HFX_CT_N;
 constexpr int kB = 8;
-constexpr int kNT = ct::PlaneThreads<kN>::value;  // threads per block of the plane kernels
+// the forward and x passes of this edge: the plane passes of hfx_ct_plane.cuh where they exist
+template <int N, bool PLANE = N % 8 == 0> struct PlanePasses;
+template <int N> struct PlanePasses<N, true> {
+  using G = ct::PlaneGeo<N>;
+  using K = ct::PlaneCfg<N>;
+  static constexpr int fwd_threads = K::fnt, x_threads = K::xnt;
+  static constexpr size_t fwd_smem = G::smem_fwd, x_smem = G::smem_x;
+  static constexpr auto fwd = ct::k_fwd_plane<N, K::fnt, K::fmb, K::un>;
+  static constexpr auto x = ct::k_x_plane<N, K::xnt, K::xmb>;
+};
+template <int N> struct PlanePasses<N, false> {
+  static constexpr int fwd_threads = ct::PlaneThreads<N>::value, x_threads = fwd_threads;
+  static constexpr size_t fwd_smem = (N * (N + 1) + ct::Plan<N>::p.twtotal) * sizeof(float2), x_smem = fwd_smem;
+  static constexpr auto fwd = ct::k_fwd_yz_ct<float, N>;
+  static constexpr auto x = ct::k_x_coulomb_ct<float, N>;
+};
+using PP = PlanePasses<kN>;
 
-cudaError_t prepare(int max_dynamic_smem, size_t smem_plane, int* blocks_fwd, int* blocks_x) {
-  const void* ks[] = {(const void*)ct::k_fwd_yz_ct<float, kN>, (const void*)ct::k_x_coulomb_ct<float, kN>,
-                      (const void*)ct::k_y_acc_dense_ct<float, kN, kB>, (const void*)ct::k_y_acc_dense_tma<float, kN, kB>,
-                      (const void*)ct::k_y_acc_diag_ct<float, kN, kB>};
+cudaError_t prepare(int max_dynamic_smem, int* blocks_fwd, int* blocks_x) {
+  const void* ks[] = {(const void*)PP::fwd, (const void*)PP::x, (const void*)ct::k_y_acc_dense_ct<float, kN, kB>,
+                      (const void*)ct::k_y_acc_dense_tma<float, kN, kB>, (const void*)ct::k_y_acc_diag_ct<float, kN, kB>};
   for (const void* k : ks) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dynamic_smem);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
   }
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_fwd, ct::k_fwd_yz_ct<float, kN>,
-                                                                kNT, smem_plane);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_fwd, PP::fwd, PP::fwd_threads, PP::fwd_smem);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_x, ct::k_x_coulomb_ct<float, kN>, kNT,
-                                                       smem_plane);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_x, PP::x, PP::x_threads, PP::x_smem);
 }
 
-void fwd_yz(int grid, size_t smem, cudaStream_t st, const float* orb, long long Ntot, const int4* couples, int c0,
-            int c1, float2* W, const float2* tw, int prefetch) {
-  ct::k_fwd_yz_ct<float, kN><<<grid, kNT, smem, st>>>(orb, Ntot, couples, c0, c1, W, tw, prefetch);
+void fwd_yz(int grid, cudaStream_t st, const float* orb, long long Ntot, const int4* couples, int c0, int c1, float2* W,
+            const float2* tw, int prefetch) {
+  PP::fwd<<<grid, PP::fwd_threads, PP::fwd_smem, st>>>(orb, Ntot, couples, c0, c1, W, tw, prefetch);
 }
 
-void x_coulomb(int grid, size_t smem, cudaStream_t st, const int4* couples, int c0, int c1, float2* W,
-               const float* vtab, const float2* tw, double* epart, int energy_only, int prefetch) {
-  ct::k_x_coulomb_ct<float, kN><<<grid, kNT, smem, st>>>(couples, c0, c1, W, vtab, tw, epart, energy_only,
-                                                                    prefetch);
+void x_coulomb(int grid, cudaStream_t st, const int4* couples, int c0, int c1, float2* W, const float* vtab,
+               const float2* tw, double* epart, int energy_only, int prefetch) {
+  PP::x<<<grid, PP::x_threads, PP::x_smem, st>>>(couples, c0, c1, W, vtab, tw, epart, energy_only, prefetch);
 }
 
 void y_acc_dense(dim3 grid, size_t smem, cudaStream_t st, const float* orb, long long Ntot, const int4* couples,
@@ -60,7 +73,7 @@ void y_acc_diag(dim3 grid, size_t smem, cudaStream_t st, const float* orb, long 
       orb, Ntot, couples, slot_list, slot_couple_base, slot_blocks, c0, W, tw, V, vscale, tmV, tma_flush);
 }
 
-const CtFns kFns = {kN, ct::DenseGeo<float, kN>::NT, &prepare, &fwd_yz, &x_coulomb, &y_acc_dense,
+const CtFns kFns = {kN, ct::DenseGeo<float, kN>::NT, PP::fwd_smem > PP::x_smem ? PP::fwd_smem : PP::x_smem, &prepare, &fwd_yz, &x_coulomb, &y_acc_dense,
                     &y_acc_dense_tma, &y_acc_diag};
 
 }  // namespace

@@ -115,7 +115,7 @@ k_y_acc_diag_ct(const T* __restrict__ orb, long long Ntot, const int4* __restric
       const int u = rest % CPI, y = rest / CPI;
       const int cr = k * CPI + u;
       const bool ok_c = ((live >> cr) & 1u) && v * PER < zcn;
-      const C* src = W + ((long long)(cs + cr - c0) * N + x) * PLANE + (long long)y * N + z0 + v * PER;
+      const C* src = W + (long long)(cs + cr - c0) * N * PLANE + x * WStride<N>::x + y * WStride<N>::y + z0 + v * PER;
       cp_async16(dstb + y * LN + u * ZC + v * PER, ok_c ? (const void*)src : (const void*)W, ok_c ? 16 : 0);
     }
     cp_async_commit();

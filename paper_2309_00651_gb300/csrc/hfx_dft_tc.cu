@@ -5,7 +5,8 @@
 // Each axis is one complex DFT of length N, written as one real GEMM with split TF32 operands:
 //   [X_re | X_im](row) = [Z_re | Z_im](row) . B,  B = [[C, -S], [S, C]] over (input, output),
 // C = cos(2 pi t f / N), S = sin(2 pi t f / N) for input index t and output frequency f, with
-// the output columns in the digit-reversed position order of the stage plan of N, so the result
+// the output columns in the digit-reversed position order of that axis's stage plan (z and y have
+// different ones, so each has its own matrix), so the result
 // lands where the x/Coulomb and inverse-y passes (hfx_ct.cuh) expect it.  The data is the A
 // operand (M = 128 rows: the plane's N lines, the rest zero), the DFT matrix B (N_mma = 2N
 // columns, K = 2N) comes pre-split (hi + lo TF32) and pre-swizzled from a table, one k-block of
@@ -14,7 +15,7 @@
 // accumulators that restart every k-block and are added, with round-to-nearest, to FP32 sums
 // (the tensor core's own accumulation rounds toward zero).
 //   z: rows y, inputs z -> P[y][f] (shared memory, FP32);
-//   y: rows f (from P, transposed as it is stored), inputs y -> registers -> W[cl][x][fy][fz].
+//   y: rows f (from P, transposed as it is stored), inputs y -> registers -> W[cl][fy][x][fz].
 // Block: 256 threads; thread 0 issues the MMAs; every mbarrier wait has an iteration limit after
 // which the block records the timeout bit in the error word, frees its TMEM and returns.
 #include <cuda_runtime.h>
@@ -203,7 +204,7 @@ k_fwd_yz_tc(const float* __restrict__ orb, long long Ntot, const int4* __restric
         *reinterpret_cast<float4*>(sah + o) = hv;
         *reinterpret_cast<float4*>(sal + o) = lv;
       }
-      copy_b(kb);
+      copy_b(KB + kb);  // y's matrix follows z's
       if (!mma_wait()) { aborted = true; break; }
 #pragma unroll
       for (int c16 = 0; c16 < NB / 32; ++c16) {
@@ -218,15 +219,15 @@ k_fwd_yz_tc(const float* __restrict__ orb, long long Ntot, const int4* __restric
       __syncthreads();
     }
     if (aborted) break;
-    // ---- W[cl][x][fy][fz]: this thread holds fz = lane row, columns jj: Re (jj < N) or Im of fy
+    // ---- W[cl][fy][x][fz]: this thread holds fz = lane row, columns jj: Re (jj < N) or Im of fy
     const int fz = 32 * q + lane;
     if (fz < N) {
-      float* wb = reinterpret_cast<float*>(W + ((long long)cl * N + x) * PLANE);
+      float* wb = reinterpret_cast<float*>(W + (long long)cl * N * PLANE + x * N);
 #pragma unroll
       for (int j = 0; j < NB / 2; ++j) {
         const int jj = h * (NB / 2) + j;
         const int fy = jj < N ? jj : jj - N;
-        wb[2 * ((long long)fy * N + fz) + (jj < N ? 0 : 1)] = acc[j];
+        wb[2 * ((long long)fy * PLANE + fz) + (jj < N ? 0 : 1)] = acc[j];
       }
     }
   }
@@ -247,7 +248,7 @@ k_fwd_yz_tc(const float* __restrict__ orb, long long Ntot, const int4* __restric
 // ------------------------------------------------------------------------------------
 bool tc_edge(int n) { return n == 32 || n == 48 || n == 64 || n == 96; }
 
-size_t tc_table_bytes(int n) { return (size_t)(2 * n / 32) * 2 * (size_t)(2 * n) * 128; }
+size_t tc_table_bytes(int n) { return (size_t)2 * (2 * n / 32) * 2 * (size_t)(2 * n) * 128; }
 
 template <int N>
 static cudaError_t prep(int* blocks) {

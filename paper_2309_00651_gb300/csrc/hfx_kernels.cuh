@@ -56,6 +56,7 @@ struct Geo {
   int n1, n2, n3;
   long long N;              // n1 n2 n3
   int S;                    // padded shared-memory row stride of the planes: n3 + 1 (odd)
+  int wx, wy;               // element strides of x and y in a couple's transform W
   DimPlan d[3];
 };
 
@@ -616,7 +617,7 @@ k_y_acc_dense(const __grid_constant__ Geo g, const T* __restrict__ orb, const in
       const int t = rest % HB, y = rest / HB;
       const int c = cs + r * HB + t;
       const bool live = !couple_empty(couples[c]) && v * PER < zcn;
-      const C* src = W + ((long long)(c - c0) * n1 + x) * plane + (long long)y * n3 + z0 + v * PER;
+      const C* src = W + (long long)(c - c0) * g.N + (long long)x * g.wx + (long long)y * g.wy + z0 + v * PER;
       cp_async16(dstb + y * LN + t * ZC + v * PER, live ? (const void*)src : (const void*)W, live ? 16 : 0);
     }
     cp_async_commit();
@@ -789,7 +790,7 @@ __device__ __forceinline__ void acc_generic_item(const Geo& g, const T* __restri
         const int t = rest % grp, y = rest / grp;
         const int c = q * grp + t;
         const bool live = c < nc && (cloc[c].x >= 0 || cloc[c].z >= 0) && v * PER < zcn;
-        const C* src = W + ((long long)(cs + c - c0) * n1 + x) * plane + (long long)y * n3 + z0 + v * PER;
+        const C* src = W + (long long)(cs + c - c0) * g.N + (long long)x * g.wx + (long long)y * g.wy + z0 + v * PER;
         cp_async16(dstb + y * LN + t * ZC + v * PER, live ? (const void*)src : (const void*)W, live ? 16 : 0);
       }
     }
