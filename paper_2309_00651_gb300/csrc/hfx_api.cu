@@ -365,6 +365,12 @@ static bool diag_available(const hfx_ctx* c) {
   return c->ct != nullptr && c->prec == HFX_PREC_FP32 && c->bsize == 8;
 }
 
+// the TMA form of the dense accumulate pass (blocks of 8; tensor maps need 16-byte row strides: FP32
+// orbital rows of an edge that is a multiple of 4), which also takes the ragged last block's pairs
+static bool ragged_dense(const hfx_ctx* c) {
+  return c->ct != nullptr && c->prec == HFX_PREC_FP32 && c->bsize == 8 && c->dense_tma && c->grid[0] % 4 == 0;
+}
+
 // Every device allocation the library makes for itself (context tables, schedules, batch tables)
 // goes through dev_alloc / dev_free: one place that counts what is held and that a test can make
 // fail (hfx_test_fail_allocation), so the error paths are exercised without exhausting a GPU.
@@ -731,12 +737,18 @@ static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 static Schedule make_host_schedule(const hfx_ctx* c, int n_orb) {
   Schedule S;
   build_schedule(S, n_orb, c->bsize, c->transform_budget, (size_t)c->N * cplx_size(c), dense_available(c),
-                 diag_available(c));
+                 diag_available(c), ragged_dense(c));
   return S;
 }
 
 // two transform buffers when the batches of a call are pipelined on the context's two streams
 static bool two_buffers(const hfx_ctx* c, const Schedule& S) { return S.nbatches > 1 && c->side && c->pipeline; }
+
+// the couple table, then for the TMA dense pass (slots of at most 32 couples) one word per slot whose set
+// bits are the couples without pairs; both start as all ones
+static size_t couple_table_bytes(const Schedule& S) {
+  return (size_t)S.max_total_couples * sizeof(int4) + (S.ragged_rows ? (size_t)S.nslots * sizeof(unsigned) : 0);
+}
 
 static Layout layout_of(const hfx_ctx* c, const Schedule& S, int n_orb, bool second_buffer) {
   Layout L;
@@ -759,7 +771,7 @@ static Layout layout_of(const hfx_ctx* c, const Schedule& S, int n_orb, bool sec
   L.W2 = take(second_buffer ? (size_t)S.max_batch_couples * c->N * cplx_size(c) : 0);
   L.epart = take((size_t)S.max_total_couples * eparts(c) * sizeof(double));
   L.eblk = take((size_t)64 * sizeof(double));  // per-block energy sums (kEnergyBlocks)
-  L.couples = take((size_t)S.max_total_couples * sizeof(int4));
+  L.couples = take(couple_table_bytes(S));
   L.total = off;
   return L;
 }
@@ -814,10 +826,13 @@ __global__ void k_cast_f32(const double* __restrict__ src, float* __restrict__ d
 }
 
 // every listed pair goes to its fixed place in the canonical couple layout of its block pair;
-// entries outside 0 <= i <= j < n_orb, and second copies of a pair, are flagged and skipped
+// entries outside 0 <= i <= j < n_orb, and second copies of a pair, are flagged and skipped.
+// dead_words (the TMA dense pass: slots of at most 32 couples) loses the bit of every couple that gets
+// a pair, and off-diagonal pairs with the last, ragged block are laid out with its orbitals as rows
 __global__ void k_plan_place(const int2* __restrict__ pairs, long long P, int n_orb, int bsize, int nb,
                              const int* __restrict__ slot_of_bp, const int* __restrict__ slot_couple_base,
-                             int4* __restrict__ couples, int* __restrict__ err) {
+                             int4* __restrict__ couples, unsigned* __restrict__ dead_words,
+                             int* __restrict__ err) {
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x) {
     const int2 ij = pairs[p];
     const int i = ij.x, j = ij.y;
@@ -828,7 +843,7 @@ __global__ void k_plan_place(const int2* __restrict__ pairs, long long P, int n_
     const int si = min(bsize, n_orb - I0), sj = min(bsize, n_orb - J0);
     int t, c;
     if (bi != bj) {
-      t = (i - I0) * sj + (j - J0);
+      t = dead_words && sj < bsize ? (j - J0) * bsize + (i - I0) : (i - I0) * sj + (j - J0);
       c = t >> 1;
     } else if (i != j) {
       const int a = i - I0, b = j - I0;  // a < b
@@ -842,6 +857,7 @@ __global__ void k_plan_place(const int2* __restrict__ pairs, long long P, int n_
     int* cp = reinterpret_cast<int*>(couples + slot_couple_base[slot] + c) + 2 * (t & 1);
     if (atomicCAS(cp, -1, i) != -1) { atomicOr(err, kErrBadPair); continue; }
     cp[1] = j;
+    if (dead_words) atomicAnd(dead_words + slot, ~(1u << c));
   }
 }
 
@@ -904,7 +920,7 @@ __global__ void k_guard_check(const char* ws, GuardSet g, int* err) {
 // places (the layout the accumulate passes assume)
 __global__ void k_check_couples(const int4* __restrict__ couples, const int* __restrict__ slot_couple_base,
                                 const int2* __restrict__ slot_blocks, int nslots, int n_orb, int bsize,
-                                int* err) {
+                                int ragged_rows, int* err) {
   for (int s = blockIdx.x; s < nslots; s += gridDim.x) {
     const int2 bp = slot_blocks[s];
     const int I0 = bp.x * bsize, J0 = bp.y * bsize;
@@ -919,7 +935,7 @@ __global__ void k_check_couples(const int4* __restrict__ couples, const int* __r
         if (ok) {
           int t, cc;
           if (bp.x != bp.y) {
-            t = (i - I0) * sj + (j - J0);
+            t = ragged_rows && sj < bsize ? (j - J0) * bsize + (i - I0) : (i - I0) * sj + (j - J0);
             cc = t >> 1;
           } else if (i != j) {
             const int a = i - I0, b = j - I0;
@@ -1026,8 +1042,7 @@ static hfx_status run_passes(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
   // the tensor maps of the TMA dense accumulate pass (one per transform buffer)
   CUtensorMap tmW[2] = {}, tmOrb = {}, tmV = {};
   bool dense_tma = false;
-  // (tensor maps need 16-byte row strides: FP32 orbital rows of an edge that is a multiple of 4)
-  if (std::is_same<T, float>::value && c->ct && S.b == 8 && c->dense_tma && !energy_only && g.n1 % 4 == 0) {
+  if (std::is_same<T, float>::value && ragged_dense(c) && S.b == 8 && !energy_only) {
     const int cpi = dense_rows_ct(g.n1) * (S.b / 2);
     dense_tma =
         encode_dense_maps(&tmW[0], Wbuf[0], S.max_batch_couples, cpi, g.wx, g.wy, &tmOrb, orb, &tmV, vacc, n_orb, g.n1) &&
@@ -1102,7 +1117,8 @@ static hfx_status run_passes(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
       const int nd = S.dense_begin[b + 1] - S.dense_begin[b];
       const int ng = S.generic_begin[b + 1] - S.generic_begin[b];
       if (nd > 0 && ct && S.b == 8 && dense_tma)  // [dense block pairs]
-        ct->y_acc_dense_tma(dim3(nzc, g.n1, nd), smem_dense_tma_ct(g.n1), st, tmW[b & 1], tmOrb, tmV, couples,
+        ct->y_acc_dense_tma(dim3(nzc, g.n1, nd), smem_dense_tma_ct(g.n1), st, tmW[b & 1], tmOrb, tmV,
+                            (const unsigned*)(couples + S.max_total_couples), n_orb,
                             S.d_dense_slots + S.dense_begin[b], S.d_slot_couple_base, S.d_slot_blocks, c0,
                             (const float2*)c->d_twct, vscale, c->d_err, (flags & HFX_TEST_STALL) ? 1 : 0);
       else if (nd > 0 && ct && S.b == 8)
@@ -1186,13 +1202,15 @@ static hfx_status stage_call(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
     HFX_CUDA_TRY(cudaMemsetAsync(vxphi, 0, (size_t)n_orb * c->N * sizeof(double), st));
   }
   int4* couples = (int4*)(ws + L.couples);
-  HFX_CUDA_TRY(cudaMemsetAsync(couples, 0xff, (size_t)S.max_total_couples * sizeof(int4), st));
+  HFX_CUDA_TRY(cudaMemsetAsync(couples, 0xff, couple_table_bytes(S), st));
   {
     const int threads = 256;
     const int blocks = (int)std::max<long long>(1, std::min<long long>((n_pairs + threads - 1) / threads,
                                                                         (long long)c->sm_count * 8));
     k_plan_place<<<blocks, threads, 0, st>>>((const int2*)pairs, n_pairs, n_orb, S.b, S.nb, S.d_slot_of_bp,
-                                             S.d_slot_couple_base, couples, c->d_err);
+                                             S.d_slot_couple_base, couples,
+                                             S.ragged_rows ? (unsigned*)(couples + S.max_total_couples) : nullptr,
+                                             c->d_err);
   }
   HFX_CUDA_TRY(cudaGetLastError());
   *orb_pass = orbitals;
@@ -1229,7 +1247,8 @@ static hfx_status apply_with(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
   if (rs != HFX_OK) return rs;
 #ifdef HFX_DEBUG
   k_check_couples<<<std::max(1, std::min(S.nslots, c->sm_count * 4)), 128, 0, st>>>(
-      (const int4*)(ws + L.couples), S.d_slot_couple_base, S.d_slot_blocks, S.nslots, n_orb, S.b, c->d_err);
+      (const int4*)(ws + L.couples), S.d_slot_couple_base, S.d_slot_blocks, S.nslots, n_orb, S.b,
+      S.ragged_rows ? 1 : 0, c->d_err);
 #endif
   if (env.prof) prof_close(c, kProfStage, e_stage, st);
   if (c->prec == HFX_PREC_FP64) rs = run_passes<double>(c, S, L, env, (const double*)orb, n_orb, flags, vxphi, st);
@@ -1662,7 +1681,8 @@ extern "C" hfx_status hfx_apply_noalloc(hfx_ctx* c, const void* orbitals, int32_
     for (int k : S.slot_cap) cap_max = std::max(cap_max, k);
     const size_t room = fixed < kNoallocScratchBytes ? kNoallocScratchBytes - fixed : 0;
     if (room >= (size_t)cap_max * couple_bytes + 256) {
-      build_schedule(S, n_orb, c->bsize, room - 256, couple_bytes, dense_available(c), diag_available(c));
+      build_schedule(S, n_orb, c->bsize, room - 256, couple_bytes, dense_available(c), diag_available(c),
+                     ragged_dense(c));
       L = layout_of(c, S, n_orb, false);
     }
   }

@@ -595,15 +595,25 @@ k_y_acc_dense_ct(const T* __restrict__ orb, long long Ntot, const int4* __restri
 // orbital tiles as two more (box ZC x N x B, landing as [orbital][y][zz]); the copies complete on
 // mbarriers that every thread waits on with a time limit.  The same boxes of the FP32 V_x phi
 // accumulator (tmV, laid out like the orbitals) are prefetched into L2 at the start, and the
-// block's scaled sums are added into them at the end by two tensor reduce-adds.  Couples without
-// pairs are read like the others (their slots of W hold stale values) and cleared in shared
-// memory before the transform.
+// block's scaled sums are added into them at the end by two tensor reduce-adds.
+//
+// Which couples hold pairs comes as one word per block pair (a set bit: couple without pairs), so
+// the row iterations of a screened list without any pair are neither copied nor transformed, and a
+// block pair without pairs ends at once; the other empty couples are read like the rest (their slots
+// of W hold stale values) and cleared in shared memory before the transform.
+//
+// A last block of fewer than B orbitals is taken as the ROW block of its block pairs (the staging
+// lays their couples out that way): its rows past n_orb are couples without pairs, the orbital tile
+// reads zeros there, and the reduce-add skips what lies outside V.  Measured:
+// 117 orbitals on 80^3, accumulate passes 7.8 -> 5.5 ms, call 19.7 -> 17.2 (the generic pass took these
+// block pairs); 96 orbitals on 128^3 with 35% of the pairs listed, 15.4 -> 10.1 ms, call 34.5 -> 30.4;
+// a full list is where it was (72^3, 128 orbitals: 3.60 -> 3.64 ms).
 constexpr long long kTmaWaitCycles = 1LL << 30;  // about half a second
 
 template <typename T, int N, int B>
 __global__ void __launch_bounds__(DenseGeo<T, N>::NT, DenseGeo<T, N>::MINB)
 k_y_acc_dense_tma(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmOrb,
-                  const __grid_constant__ CUtensorMap tmV, const int4* __restrict__ couples,
+                  const __grid_constant__ CUtensorMap tmV, const unsigned* __restrict__ dead_words, int n_orb,
                   const int* __restrict__ slot_list, const int* __restrict__ slot_couple_base, const int2* __restrict__ slot_blocks, int c0,
                   const cx<T>* __restrict__ twg, double vscale, int* __restrict__ err, int stall) {
   using C = cx<T>;
@@ -619,14 +629,14 @@ k_y_acc_dense_tma(const __grid_constant__ CUtensorMap tmW, const __grid_constant
   constexpr uint32_t kOrbTileBytes = B * PTS * sizeof(T);
   constexpr StagePlan P = Plan<N>::p;
   static_assert(B % RPI == 0, "rows per iteration must divide the block");
-  static_assert(B * HB <= 32, "one mask word per block pair");
+  static_assert(B * HB == 32, "one mask word per block pair");
+  constexpr unsigned kItMask = CPI == 32 ? ~0u : (1u << (CPI & 31)) - 1u;  // the couples of one iteration
   static_assert(kTileBytes % 128 == 0 && kOrbTileBytes % 128 == 0, "tensor-copy destinations stay 128-byte aligned");
   // the host encodes boxes of 16 x couples x N (transforms) and 8 x N x 8 (orbitals): the byte
   // counts the mbarriers expect are those boxes only when ZC = 8 and B = 8
   static_assert(ZC == 8 && B == 8, "box sizes of the host's tensor maps");
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bars[RING + 1];  // the ring's slots, then the orbital tiles
-  __shared__ unsigned live_mask;
   unsigned char* base = smem_raw + ((128u - (tc::smem_u32(smem_raw) & 127u)) & 127u);
   C* tiles = reinterpret_cast<C*>(base);                   // RING x [N][LN]
   T* phiI = reinterpret_cast<T*>(tiles + RING * N * LN);   // [B][PTS]
@@ -640,23 +650,34 @@ k_y_acc_dense_tma(const __grid_constant__ CUtensorMap tmW, const __grid_constant
   const int x = blockIdx.y;
   const int slot = slot_list[blockIdx.z];
   const int2 blk = slot_blocks[slot];
-  const int I0 = blk.x * B, J0 = blk.y * B;
+  const bool ragged = blk.y * B + B > n_orb;  // the last block has fewer orbitals: it gives the rows
+  const int I0 = (ragged ? blk.y : blk.x) * B, J0 = (ragged ? blk.x : blk.y) * B;
   const int cs = slot_couple_base[slot];
+  const unsigned dead_all = dead_words[slot];
+  // the iterations with pairs, in order: bit k for rows k RPI .. k RPI + RPI - 1
+  unsigned todo = 0;
+#pragma unroll
+  for (int k = 0; k < ITERS; ++k)
+    if (((dead_all >> (k * CPI)) & kItMask) != kItMask) todo |= 1u << k;
+  if (todo == 0) return;  // the same for every thread of the block
   // thread 0's account of its copies: couple tiles issued, tiles it has seen land (in order), and
   // whether the orbital tiles have landed; what it has not seen land is waited for before exit
   int issued = 0, landed = 0;
   bool orb_landed = false;
-  // iteration k's couple tile -> ring slot k % RING (thread 0 only).  stall (a failure-detection
+  unsigned to_issue = todo;
+  // the next iteration's couple tile -> the next ring slot (thread 0 only).  stall (a failure-detection
   // test): the first tile's mbarrier expects 16 bytes more than the copy brings, so its wait can
   // only end by running out
-  auto issue = [&](int k) {
-    if (k >= ITERS) return;
-    uint64_t* bar = &bars[k % RING];
-    tma::expect_tx(bar, kTileBytes + (stall && k == 0 ? 16u : 0u));
-    tma::load4d(tiles + (k % RING) * N * LN, mapW, 2 * z0, cs - c0 + k * CPI, 0, x, bar);
-    issued = k + 1;
+  auto issue = [&]() {
+    if (to_issue == 0) return;
+    const int k = __ffs(to_issue) - 1;
+    to_issue &= to_issue - 1;
+    uint64_t* bar = &bars[issued % RING];
+    tma::expect_tx(bar, kTileBytes + (stall && issued == 0 ? 16u : 0u));
+    tma::load4d(tiles + (issued % RING) * N * LN, mapW, 2 * z0, cs - c0 + k * CPI, 0, x, bar);
+    ++issued;
   };
-  // thread 0 starts the copies at once: they do not depend on which couples hold pairs
+  // thread 0 starts the copies at once
   __shared__ int skip;
   __shared__ int failed;  // set by any thread whose wait ran out; read after the next barrier
   if (threadIdx.x == 0) {
@@ -670,21 +691,15 @@ k_y_acc_dense_tma(const __grid_constant__ CUtensorMap tmW, const __grid_constant
       tma::load4d(phiI, mapOrb, z0, 0, I0, x, &bars[RING]);
       tma::load4d(accI, mapOrb, z0, 0, J0, x, &bars[RING]);
 #pragma unroll
-      for (int k = 0; k < RING - 1; ++k) issue(k);
+      for (int k = 0; k < RING - 1; ++k) issue();
       // the V_x phi tiles that the flush reads and rewrites at the end head for L2 now
       tma::prefetch4d(&tmV, z0, 0, I0, x);
       tma::prefetch4d(&tmV, z0, 0, J0, x);
     }
   }
-  // which couples of the block pair hold pairs (bit t of the mask: couple cs + t)
-  if (threadIdx.x < 32) {
-    const unsigned m = __ballot_sync(0xffffffffu, threadIdx.x < B * HB && !couple_empty(couples[cs + threadIdx.x]));
-    if (threadIdx.x == 0) live_mask = m;
-  }
   for (int i = threadIdx.x; i < P.twtotal; i += NT) tw[i] = twg[i];
   __syncthreads();
   if (skip) return;  // the same for every thread of the block
-  const unsigned live = live_mask;
 
   // a wait that runs out is retried once (the copy may still land); after that this thread waits
   // no more, and the block stops at its next vote
@@ -718,14 +733,28 @@ k_y_acc_dense_tma(const __grid_constant__ CUtensorMap tmW, const __grid_constant
   // every thread's waits so far have ended with their copies landed: the same verdict for the block
   __syncthreads();
   bool block_ok = *(volatile int*)&failed == 0;
-  // (a constant trip count, so the loop unrolls; after a failed vote the iterations do nothing)
+  // rows of skipped iterations add nothing to V_I
+  if (todo != (1u << ITERS) - 1u) {
 #pragma unroll
-  for (int kk = 0; kk < ITERS; ++kk) {
-    if (!block_ok) continue;
-    if (threadIdx.x == 0) issue(kk + RING - 1);
-    C* buf = tiles + (kk % RING) * N * LN;
-    if (wait(&bars[kk % RING], (uint32_t)((kk / RING) & 1))) landed = kk + 1;
-    const unsigned dead = (~live >> (kk * CPI)) & ((1u << CPI) - 1u);
+    for (int k = 0; k < NP; ++k) {
+      const int p = threadIdx.x + k * NT;
+      if (p >= PTS) continue;
+      for (int r = 0; r < B; ++r)
+        if (!((todo >> (r / RPI)) & 1u)) accI[r * PTS + p] = T(0);
+    }
+  }
+  unsigned rest = todo;
+  // (a constant trip count, so the loop unrolls and the ring slots are constants; past the last
+  // iteration, and after a failed vote, the rounds do nothing)
+#pragma unroll
+  for (int n = 0; n < ITERS; ++n) {
+    if (rest == 0 || !block_ok) continue;
+    const int kk = __ffs(rest) - 1;
+    rest &= rest - 1;
+    if (threadIdx.x == 0) issue();
+    C* buf = tiles + (n % RING) * N * LN;
+    if (wait(&bars[n % RING], (uint32_t)((n / RING) & 1))) landed = n + 1;
+    const unsigned dead = (dead_all >> (kk * CPI)) & kItMask;
     if (dead) {  // the same for every thread of the block
       for (int i = threadIdx.x; i < N * LN; i += NT)
         if ((dead >> ((i / ZC) % CPI)) & 1u) buf[i] = C{};

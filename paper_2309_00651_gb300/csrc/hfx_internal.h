@@ -72,10 +72,12 @@ struct CtFns {
   // the same pass with its tiles moved by TMA: tmW maps the batch's transform buffer (dimensions
   // z reals, couple, y, x), tmOrb the FP32 orbitals and tmV the FP32 accumulator V (both z, y,
   // orbital, x), into which the pass adds by tensor reduce-adds; boxes as k_y_acc_dense_tma reads
-  // them, shared memory smem_dense_ct + 128; stall:
+  // them, shared memory smem_dense_ct + 128; dead_words: per slot, the couples without pairs; a slot
+  // whose second block is the last, ragged one has its couples laid out with that block's orbitals as
+  // rows; stall:
   // the HFX_TEST_STALL failure-detection test (each block's first wait runs out)
   void (*y_acc_dense_tma)(dim3 grid, size_t smem, cudaStream_t st, const CUtensorMap& tmW, const CUtensorMap& tmOrb,
-                          const CUtensorMap& tmV, const int4* couples, const int* slot_list,
+                          const CUtensorMap& tmV, const unsigned* dead_words, int n_orb, const int* slot_list,
                           const int* slot_couple_base, const int2* slot_blocks, int c0, const float2* tw,
                           double vscale, int* err, int stall);
   // full diagonal block pairs (B = 8), same arguments and threads as the dense pass; tma_flush:

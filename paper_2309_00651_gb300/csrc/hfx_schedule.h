@@ -26,6 +26,7 @@ struct Schedule {
   // per batch: slots taken by the dense accumulation kernel and by the generic one
   std::vector<int> dense_slots, generic_slots, diag_slots;  // concatenated over batches
   std::vector<int> dense_begin, generic_begin, diag_begin;  // [nbatches + 1] offsets into the lists
+  bool ragged_rows = false;             // layout of ragged off-diagonal block pairs (build_schedule)
   long long max_batch_couples = 0, max_total_couples = 0;
   // device copies
   int2* d_slot_blocks = nullptr;
@@ -39,14 +40,18 @@ struct Schedule {
 static int block_size_of(int bi, int b, int n_orb) { return std::min(b, n_orb - bi * b); }
 
 // couples of a slot in the canonical layout: I != J: all sI sJ pairs, couple t/2 of
-// t = (i - I0) sJ + (j - J0); I == J: the sI (sI-1)/2 pairs i < j first, then the sI diagonal ones.
+// t = (i - I0) sJ + (j - J0), or of t = (j - J0) sI + (i - I0) where the last, ragged block gives the
+// rows (ragged_rows; sI is even there); I == J: the sI (sI-1)/2 pairs i < j first, then the sI diagonal ones.
 static int slot_capacity(int si, int sj, bool diag) {
   if (!diag) return (si * sj + 1) / 2;
   return (si * (si - 1) / 2 + 1) / 2 + (si + 1) / 2;
 }
 
+// ragged_ok: the dense pass also takes block pairs (full block, last block of fewer orbitals), whose
+// couples are then laid out with the last block's orbitals as rows
 static void build_schedule(Schedule& S, int n_orb, int b, size_t transform_budget, size_t bytes_per_couple,
-                           bool dense_ok, bool diag_ok) {
+                           bool dense_ok, bool diag_ok, bool ragged_ok = false) {
+  S.ragged_rows = ragged_ok;
   S.n_orb = n_orb;
   S.b = b;
   S.nb = (n_orb + b - 1) / b;
@@ -117,7 +122,7 @@ static void build_schedule(Schedule& S, int n_orb, int b, size_t transform_budge
     for (int k = S.batch_slot_begin[bt]; k < S.batch_slot_begin[bt + 1]; ++k) {
       const int2 bp = S.slot_blocks[k];
       const bool full = block_size_of(bp.x, b, n_orb) == b && block_size_of(bp.y, b, n_orb) == b;
-      if (dense_ok && bp.x != bp.y && full) S.dense_slots.push_back(k);
+      if (dense_ok && bp.x != bp.y && (full || ragged_ok)) S.dense_slots.push_back(k);
       else if (diag_ok && bp.x == bp.y && full) S.diag_slots.push_back(k);
       else S.generic_slots.push_back(k);
     }
