@@ -158,24 +158,26 @@ typedef struct {
 } hfx_apply_args;
 
 /* hfx_apply_batched -- several independent problems (each with its own context, so its own
- * cell, grid, orbital count and workspace), all their passes in ONE persistent launch: the
- * uneven batch of independent configurations, distributed as independent work the way Sec. 2.2
- * spreads independent work over processor groups.
- *   Per problem the call first enqueues its staging (V_x phi cleared, pairs placed, the FP32
- *   orbital copy), then one launch runs every pass of every problem from a device work queue:
- *   items (planes, tiles) are taken in a fixed task order by all blocks; the tasks of one problem
- *   run as a chain (forward, x/Coulomb and accumulate pass of each batch of couples, then the
- *   energy sum) and the chains of different problems are interleaved, so the problems share the
- *   GPU.  A block whose item depends on an unfinished task waits for it at most the context's
- *   wait budget (hfx_set_wait_budget); a wait that runs out sets HFX_ERR_TIMEOUT in the error
- *   word of that problem's context, every block then stops, and the call's results are undefined.
- *   Results equal hfx_apply's up to rounding order (the batched passes are the runtime-geometry
- *   forms for every grid).
+ * cell, grid, orbital count and workspace) sharing the GPU: the uneven batch of independent
+ * configurations, distributed as independent work the way Sec. 2.2 spreads independent work over
+ * processor groups.
+ *   Problems that are all small (one orbital block each and less work than a call's launches take)
+ *   run in ONE persistent launch: per problem the call first enqueues its staging (V_x phi cleared,
+ *   pairs placed, the FP32 orbital copy), then one launch runs every pass of every problem from a
+ *   device work queue: items (planes, tiles) are taken in a fixed task order by all blocks; the
+ *   tasks of one problem run as a chain (forward, x/Coulomb and accumulate pass of each batch of
+ *   couples, then the energy sum) and the chains of different problems are interleaved.  A block
+ *   whose item depends on an unfinished task waits for it at most the context's wait budget
+ *   (hfx_set_wait_budget); a wait that runs out sets HFX_ERR_TIMEOUT in the error word of that
+ *   problem's context, every block then stops, and the call's results are undefined.
+ *   Otherwise each problem runs the passes of hfx_apply on its context's own stream, forked from
+ *   cuda_stream and joined to it, so that the problems fill each other's gaps.
+ *   Results equal hfx_apply's up to rounding order.  Both forms can be captured in a CUDA graph.
  *   Rules: same argument rules per problem as hfx_apply; one distinct context per problem; every
  *   context needs the same precision and device and planes that fit in shared memory
  *   (HFX_ERR_UNSUPPORTED_GRID otherwise); each context's workspace must hold hfx_workspace_bytes
- *   for its problem; batched calls led by one context must not overlap on the GPU.  The queue tables live in a
- *   device buffer owned by the first context (ctxs[0]); the first call that needs a larger one
+ *   for its problem; batched calls led by one context must not overlap on the GPU.  The persistent form's
+ *   queue tables live in a device buffer owned by the first context (ctxs[0]); the first call that needs a larger one
  *   allocates it (and synchronises the stream), so make that call before any stream capture --
  *   during capture such a call is rejected with HFX_ERR_INVALID_ARG.  Stops at the first problem
  *   whose arguments are rejected and returns that error. */

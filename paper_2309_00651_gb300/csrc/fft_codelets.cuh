@@ -16,6 +16,8 @@ namespace hfx {
 template <typename T> struct cx_t;
 template <> struct cx_t<float> { using type = float2; };
 template <> struct cx_t<double> { using type = double2; };
+// a complex FP32 value whose adds go two components an instruction (cadd and csub below)
+struct __align__(8) cpair { float x, y; };
 template <typename T> using cx = typename cx_t<T>::type;
 
 template <typename C> __host__ __device__ __forceinline__ C mk(decltype(C::x) a, decltype(C::x) b) {
@@ -32,24 +34,25 @@ template <typename C> __device__ __forceinline__ C cmulc(C a, C b) {
   return mk<C>(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
 }
 // FP32 pairs in one instruction (add.f32x2 and so on round each half like the scalar instruction): the
-// FMA pipe takes them at the same rate per element, but they need half the issue slots, which bound the
-// plane passes
-__device__ __forceinline__ unsigned long long pack2(float2 a) {
+// FMA pipe takes them at the same rate per element, but they need half the issue slots.  The plane passes
+// (cpair) gain 3 to 5% from it (72^3, 256 couples: forward 296 -> 288 us, x pass 395 -> 377); the
+// runtime-geometry and accumulate passes lose 1 to 4% (register pairs) and keep float2.
+__device__ __forceinline__ unsigned long long pack2(cpair a) {
   unsigned long long r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
   return r;
 }
-__device__ __forceinline__ float2 unpack2(unsigned long long a) {
-  float2 r;
+__device__ __forceinline__ cpair unpack2(unsigned long long a) {
+  cpair r;
   asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
   return r;
 }
-template <> __device__ __forceinline__ float2 cadd<float2>(float2 a, float2 b) {
+template <> __device__ __forceinline__ cpair cadd<cpair>(cpair a, cpair b) {
   unsigned long long r;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
   return unpack2(r);
 }
-template <> __device__ __forceinline__ float2 csub<float2>(float2 a, float2 b) {
+template <> __device__ __forceinline__ cpair csub<cpair>(cpair a, cpair b) {
   unsigned long long r;
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
   return unpack2(r);
@@ -66,13 +69,6 @@ template <int S, typename C> __device__ __forceinline__ C cfma_si(C a, C b, decl
 template <typename C> __device__ __forceinline__ C cfma(C a, C b, decltype(C::x) c) {
   return mk<C>(a.x + c * b.x, a.y + c * b.y);
 }
-#ifdef PACKFMA
-template <> __device__ __forceinline__ float2 cfma<float2>(float2 a, float2 b, float c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack2(b)), "l"(pack2(make_float2(c, c))), "l"(pack2(a)));
-  return unpack2(r);
-}
-#endif
 // s * i * a, s = +-1 (compile time)
 template <int S, typename C> __device__ __forceinline__ C mul_si(C a) {
   if constexpr (S > 0) return mk<C>(-a.y, a.x);
@@ -282,6 +278,18 @@ template <int DIR, typename C> struct Dft<12, DIR, C> {
 };
 template <int DIR, typename C> struct Dft<16, DIR, C> {
   static __device__ __forceinline__ void run(C (&x)[16]) { dft_composite<4, 4, DIR>(x); }
+};
+template <int DIR, typename C> struct Dft<15, DIR, C> {
+  static __device__ __forceinline__ void run(C (&x)[15]) { dft_coprime<3, 5, DIR>(x); }
+};
+template <int DIR, typename C> struct Dft<25, DIR, C> {
+  static __device__ __forceinline__ void run(C (&x)[25]) { dft_composite<5, 5, DIR>(x); }
+};
+template <int DIR, typename C> struct Dft<27, DIR, C> {
+  static __device__ __forceinline__ void run(C (&x)[27]) { dft_composite<3, 9, DIR>(x); }
+};
+template <int DIR, typename C> struct Dft<30, DIR, C> {
+  static __device__ __forceinline__ void run(C (&x)[30]) { dft_coprime<2, 15, DIR>(x); }
 };
 template <int DIR, typename C> struct Dft<18, DIR, C> {
   static __device__ __forceinline__ void run(C (&x)[18]) { dft_coprime<2, 9, DIR>(x); }

@@ -41,6 +41,15 @@ __host__ __device__ constexpr Factors best_factors(int n) {
   return best;
 }
 
+// A large radix R of the plane passes (hfx_ct_plane.cuh) as two consecutive stages of the radices above
+// (b = 1: it is one of them): the digit-reversed place of its output k is (k mod a) b + k / a.
+struct PlaneRadices { int a, b; };
+__host__ __device__ constexpr PlaneRadices plane_radices(int R) {
+  return R == 15 ? PlaneRadices{5, 3} : R == 18 ? PlaneRadices{9, 2} : R == 20 ? PlaneRadices{10, 2}
+       : R == 24 ? PlaneRadices{12, 2} : R == 25 ? PlaneRadices{5, 5} : R == 27 ? PlaneRadices{9, 3}
+       : R == 30 ? PlaneRadices{10, 3} : R == 32 ? PlaneRadices{16, 2} : PlaneRadices{R, 1};
+}
+
 // Per-stage data of one length: radices, sub-lengths m[s] = n / (r[0] ... r[s]) and the offset of
 // stage s's twiddle table [m][r] (w_L^{j1 k}, L = r m; stages with m = 1 have none).
 struct StagePlan {

@@ -316,15 +316,15 @@ static std::vector<double> stage_twiddles(int n) {
 }
 
 // the edges whose forward and x passes are the plane passes (hfx_ct_plane.cuh): z and x split (n / 4) x 4
-static bool plane_edge(int n) { return n % 8 == 0; }
+static bool plane_edge(int n) { return n % 4 == 0; }
 
 // twiddles of the forward and x passes of edge n: w_n^{e k}, e < 4, k < n / 4 at ((k / 2) 4 + e) 2 + k % 2,
 // then y's first stage [j][k]; the stage tables where the passes run one stage at a time
 static std::vector<double> plane_twiddles(int n) {
   if (!plane_edge(n)) return stage_twiddles(n);
   const StagePlan y = stage_plan(n);
-  const int R = n / 4;
-  std::vector<double> tw(2 * (size_t)(4 * R + y.r[0] * y.m[0]));
+  const int R = n / 4, R2 = R + R % 2;
+  std::vector<double> tw(2 * (size_t)(4 * R2 + y.r[0] * y.m[0]));
   for (int e = 0; e < 4; ++e)
     for (int k = 0; k < R; ++k) {
       const cs_pair w = cossin_2pi_frac((long long)e * k, n);
@@ -333,19 +333,22 @@ static std::vector<double> plane_twiddles(int n) {
       tw[2 * idx + 1] = -w.s;
     }
   const std::vector<double> ty = stage_twiddles(n);
-  std::copy_n(ty.begin(), 2 * (size_t)(y.r[0] * y.m[0]), tw.begin() + 2 * (size_t)(4 * R));
+  std::copy_n(ty.begin(), 2 * (size_t)(y.r[0] * y.m[0]), tw.begin() + 2 * (size_t)(4 * R2));
   return tw;
 }
 
-// the split of z and x of a plane edge
+// the split of z and x of a plane edge: n / 4 (as the two radices whose order it keeps) x 4
 static void set_plane_plan(DimPlan& d) {
-  d.ns = 2;
-  d.r[0] = d.n / 4;
-  d.m[0] = 4;
-  d.r[1] = 4;
-  d.m[1] = 1;
-  for (int s = 2; s < kMaxStages; ++s) { d.r[s] = 1; d.m[s] = 1; }
-  for (int s = 0; s < kMaxStages; ++s) d.mdiv[s] = FastDiv::make((uint32_t)d.m[s]);
+  const PlaneRadices p = plane_radices(d.n / 4);
+  const int r[3] = {p.a, p.b > 1 ? p.b : 4, 4};
+  d.ns = p.b > 1 ? 3 : 2;
+  int m = d.n;
+  for (int s = 0; s < kMaxStages; ++s) {
+    d.r[s] = s < d.ns ? r[s] : 1;
+    m = s < d.ns ? m / r[s] : 1;
+    d.m[s] = m;
+    d.mdiv[s] = FastDiv::make((uint32_t)m);
+  }
 }
 
 // pencil kernels: rows blocks of rb rows (padded stride n3 + 1) and single z-chunk columns
@@ -1015,6 +1018,7 @@ struct CallEnv {
   char* ws;
   cudaStream_t side;
   bool prof;
+  bool simt_fwd = false;  // HFX_PREC_MIXED_TC contexts: the FP32 forward pass (batched calls)
 };
 
 template <typename T>
@@ -1084,7 +1088,7 @@ static hfx_status run_passes(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
         Passes<T>::inv_z_rows(g, gr, smem_rows(c, c->rb), fs, couples, c0, c1, c->rb, W, (const C*)c->d_tw[2]);
       close(kProfX, e0, fs);
     } else {
-      if (ct && c->tc_dft) {
+      if (ct && c->tc_dft && !env.simt_fwd) {
         const int gt = (int)std::min<long long>(items1, (long long)c->sm_count * c->blocks_fwd_tc);
         dft::fwd_yz_tc(g.n1, std::max(gt, 1), fs, (const float*)orb, g.N, couples, c0, c1, (float2*)W,
                        (const unsigned char*)c->d_dftb, c->d_err);
@@ -1354,6 +1358,8 @@ static hfx_status batched_persistent(hfx_ctx* const* ctxs, const hfx_apply_args*
     BatchProblem<T> P;
     std::memset(&P, 0, sizeof(P));
     P.g = c->geo;
+    P.g.wx = P.g.n2 * P.g.n3;  // the runtime-geometry items keep W as [couple][x][y][z]
+    P.g.wy = P.g.n3;
     P.orb = (const T*)orb;
     P.couples = (const int4*)(env.ws + L.couples);
     P.W = (cx<T>*)(env.ws + L.W);
@@ -1370,8 +1376,6 @@ static hfx_status batched_persistent(hfx_ctx* const* ctxs, const hfx_apply_args*
     P.tw3 = (const cx<T>*)c->d_tw[2];
     P.slot_couple_base = S->d_slot_couple_base;
     P.slot_blocks = S->d_slot_blocks;
-    P.twct = (const cx<T>*)c->d_twplane;
-    P.ct_n = std::is_same<T, float>::value && c->ct ? c->grid[0] : 0;
     P.err = c->d_err;
     P.vscale = -c->alpha / (double)c->N;
     P.escale = -0.5 * c->alpha * c->omega / ((double)c->N * (double)c->N);
@@ -1409,7 +1413,7 @@ static hfx_status batched_persistent(hfx_ctx* const* ctxs, const hfx_apply_args*
     if (std::is_same<T, float>::value && !eo) add(kTaskWiden, (P.n_v + kWidenPerItem - 1) / kWidenPerItem, 0, 0, 0);
     add(kTaskEnergy, 1, 0, 0, 0);
     chains.push_back(ch);
-    smem = std::max(smem, P.ct_n ? c->ct->smem_plane : std::max(smem_fwd(c), smem_x(c)));
+    smem = std::max({smem, smem_fwd(c), smem_x(c)});
   }
   if (probs.empty()) return HFX_OK;
   // the accumulate tiles take at most the planes' footprint (largest couple group and orbital
@@ -1481,6 +1485,61 @@ static hfx_status batched_persistent(hfx_ctx* const* ctxs, const hfx_apply_args*
   return HFX_OK;
 }
 
+// Whether every problem of a batch is so small that the persistent launch is the faster form: a single
+// orbital block (one chain of three passes) and next to no work (n_orb (n_orb + 1) / 2 pairs x N points;
+// FP64 takes about 30 times FP32's time for it).  Measured, FP32, one persistent launch / forked streams /
+// one call each in a row, us: 8 problems of 2-4 orbitals on 24^3 211 / 233 / 472, 24 of them 551 / 563 /
+// 1370, but 8 of 4-8 on 24^3 and 30^3 351 / 265 / 538, 24 of them 946 / 613 / 1606, and 6 of 24-72 on
+// 48^3 to 64^3 29200 / 8700 / 9200 (its items are the runtime-geometry ones and the generic accumulate
+// tile, and a task waits for the whole task before it).
+static bool batch_is_small(hfx_ctx* const* ctxs, const hfx_apply_args* args, int32_t n) {
+  for (int32_t k = 0; k < n; ++k) {
+    const double work = 0.5 * args[k].n_orb * (args[k].n_orb + 1.0) * (double)ctxs[k]->N;
+    if (args[k].n_orb > ctxs[k]->bsize || work > (ctxs[k]->prec == HFX_PREC_FP64 ? 7e3 : 2e5)) return false;
+  }
+  return true;
+}
+
+// The batch as one evaluation per problem, each with its own passes on its context's second stream, forked
+// from the caller's stream and joined to it: launches of different problems fill each other's tails.
+// Everything that can be refused is refused before anything is enqueued.
+static hfx_status batched_forked(hfx_ctx* const* ctxs, const hfx_apply_args* args, int32_t n, cudaStream_t st) {
+  std::vector<Schedule*> scheds(n, nullptr);
+  for (int32_t k = 0; k < n; ++k) {
+    hfx_ctx* c = ctxs[k];
+    if (c->pencil)
+      return fail(HFX_ERR_UNSUPPORTED_GRID, "problem %d: planes exceed shared memory (use hfx_apply_sequential)", (int)k);
+    if (args[k].n_pairs == 0) continue;
+    const size_t planes = std::max(smem_fwd(c), smem_x(c));
+    if (planes + 1024 > (size_t)c->max_smem)  // (the limit of the persistent form)
+      return fail(HFX_ERR_UNSUPPORTED_GRID, "a batch tile needs %zu bytes of shared memory (limit %d)", planes, c->max_smem);
+    hfx_status s = get_schedule(c, args[k].n_orb, &scheds[k]);
+    if (s != HFX_OK) return s;
+    const size_t need = layout_of(c, *scheds[k], args[k].n_orb, false).total;
+    if (!c->ws || c->ws_bytes < need)
+      return fail(HFX_ERR_OOM, "problem %d: workspace too small: have %zu bytes, need %zu", (int)k, c->ws_bytes, need);
+  }
+  hfx_status result = HFX_OK;
+  HFX_CUDA_TRY(cudaEventRecord(ctxs[0]->ev_fork, st));
+  for (int32_t k = 0; k < n && result == HFX_OK; ++k) {
+    hfx_ctx* c = ctxs[k];
+    const hfx_apply_args& a = args[k];
+    if (!scheds[k]) {
+      result = apply_empty(c, a.n_orb, a.flags, a.ex_dev, a.vxphi, st);
+      continue;
+    }
+    HFX_CUDA_TRY(cudaStreamWaitEvent(c->side, ctxs[0]->ev_fork, 0));
+    CallEnv env{(char*)c->ws, nullptr, false};
+    env.simt_fwd = true;
+    result = apply_with(c, *scheds[k], layout_of(c, *scheds[k], a.n_orb, false), env, a.orbitals, a.n_orb, a.pairs,
+                        a.n_pairs, a.flags, a.ex_dev, a.vxphi, c->side);
+    // joined also after a failed launch: the caller's stream (or its capture) waits for what was enqueued
+    HFX_CUDA_TRY(cudaEventRecord(c->ev_p2, c->side));
+    HFX_CUDA_TRY(cudaStreamWaitEvent(st, c->ev_p2, 0));
+  }
+  return result;
+}
+
 extern "C" hfx_status hfx_apply_batched(hfx_ctx* const* ctxs, const hfx_apply_args* args, int32_t n, void* cuda_stream) {
   g_last_error.clear();
   if (n < 0 || (n > 0 && (!ctxs || !args))) return fail(HFX_ERR_INVALID_ARG, "bad batch arguments");
@@ -1502,6 +1561,9 @@ extern "C" hfx_status hfx_apply_batched(hfx_ctx* const* ctxs, const hfx_apply_ar
     if (std::adjacent_find(seen.begin(), seen.end()) != seen.end())
       return fail(HFX_ERR_INVALID_ARG, "a context appears twice in the batch (each problem needs its own)");
   }
+  bool stall = false;  // a failure-detection test makes a wait of the persistent launch run out
+  for (int32_t k = 0; k < n; ++k) stall |= (args[k].flags & HFX_TEST_STALL) != 0;
+  if (!stall && !batch_is_small(ctxs, args, n)) return batched_forked(ctxs, args, n, (cudaStream_t)cuda_stream);
   hfx_status s = ctxs[0]->prec == HFX_PREC_FP64 ? batched_persistent<double>(ctxs, args, n, (cudaStream_t)cuda_stream)
                                                 : batched_persistent<float>(ctxs, args, n, (cudaStream_t)cuda_stream);
   return s;

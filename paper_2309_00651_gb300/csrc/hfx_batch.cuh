@@ -1,5 +1,7 @@
 // One persistent launch for a batch of independent exchange problems (cells, grids and orbital
-// counts may all differ).
+// counts may all differ): the form of hfx_apply_batched for problems so small that a call of their own
+// is mostly launches (batch_is_small in hfx_api.cu; larger ones run their own passes on forked streams).
+// Every item here is a runtime-geometry one.
 //
 // Work is a list of tasks; a task is one pass of one batch of pair couples of one problem (the
 // forward plane pass, the x/Coulomb pass or the inverse-y accumulate pass) or the final energy
@@ -22,7 +24,6 @@
 #include <type_traits>
 
 #include "hfx_ct.cuh"
-#include "hfx_ct_plane.cuh"
 #include "hfx_kernels.cuh"
 
 namespace hfx {
@@ -49,66 +50,10 @@ struct BatchProblem {
   const cx<T>* tw3;
   const int* slot_couple_base;
   const int2* slot_blocks;
-  const cx<T>* twct;            // twiddles of the compile-time forward and x passes (ct_n > 0)
   int* err;                     // the problem's context error word
   double vscale, escale;
   int n_orb, bsize, grp, phi_smem, cap_max, total_couples, accumulate, energy_only;
-  int ct_n;                     // cubic FP32 edge with compile-time forward and x passes, else 0
 };
-
-// forward / x item of an FP32 problem through the compile-time passes of its edge; false when the
-// problem has none (the runtime-geometry item runs instead)
-// (tw_ok: the twiddle table of edge N is already in shared memory from this block's previous item)
-template <typename T, int N>
-__device__ __forceinline__ bool ct_item_n(const BatchProblem<T>& P, int kind, int a0, long long local,
-                                          unsigned char* smem_raw, float (*redf)[32], int par, bool tw_ok) {
-  if constexpr (std::is_same<T, float>::value) {
-    if (P.ct_n != N) return false;
-    if constexpr (N % 8 == 0) {
-      using G = ct::PlaneGeo<N>;
-      float2* tw = reinterpret_cast<float2*>(smem_raw);
-      float2* buf = tw + G::TW + G::TWY;
-      if (!tw_ok) {
-        for (int i = threadIdx.x; i < G::TW + G::TWY; i += blockDim.x) tw[i] = P.twct[i];
-        __syncthreads();
-      }
-      const int cl = (int)local / N, pl = (int)local - cl * N;
-      const int4 cp = P.couples[a0 + cl];
-      if (couple_empty(cp)) return true;
-      if (kind == kTaskFwd)
-        ct::fwd_plane_item<N, kThreadsBatch, 2>(P.orb, P.g.N, cp, P.W, buf, tw, cl, pl);
-      else
-        ct::x_plane_item<N, kThreadsBatch>(a0, P.W, P.vtab, P.epart, P.energy_only, buf, tw, redf, par, cl, pl);
-    } else {
-      constexpr StagePlan SP = ct::Plan<N>::p;
-      float2* buf = reinterpret_cast<float2*>(smem_raw);
-      float2* tw = buf + N * (N + 1);
-      if (!tw_ok)
-        for (int i = threadIdx.x; i < SP.twtotal; i += blockDim.x) tw[i] = P.twct[i];
-      if (kind == kTaskFwd)
-        ct::fwd_yz_ct_item<float, N>(P.orb, P.g.N, P.couples, a0, P.W, buf, tw, (int)local);
-      else
-        ct::x_coulomb_ct_item<float, N>(P.couples, a0, P.W, P.vtab, P.epart, P.energy_only, buf, tw, redf, par,
-                                        (int)local);
-    }
-    return true;
-  } else {
-    return false;
-  }
-}
-
-template <typename T>
-__device__ __forceinline__ bool ct_item(const BatchProblem<T>& P, int kind, int a0, long long local,
-                                        unsigned char* smem_raw, float (*redf)[32], int par, bool tw_ok) {
-  return ct_item_n<T, 32>(P, kind, a0, local, smem_raw, redf, par, tw_ok) ||
-         ct_item_n<T, 48>(P, kind, a0, local, smem_raw, redf, par, tw_ok) ||
-         ct_item_n<T, 64>(P, kind, a0, local, smem_raw, redf, par, tw_ok) ||
-         ct_item_n<T, 72>(P, kind, a0, local, smem_raw, redf, par, tw_ok) ||
-         ct_item_n<T, 80>(P, kind, a0, local, smem_raw, redf, par, tw_ok) ||
-         ct_item_n<T, 90>(P, kind, a0, local, smem_raw, redf, par, tw_ok) ||
-         ct_item_n<T, 96>(P, kind, a0, local, smem_raw, redf, par, tw_ok) ||
-         ct_item_n<T, 128>(P, kind, a0, local, smem_raw, redf, par, tw_ok);
-}
 
 struct BatchTask {
   long long first;  // number of this task's first item
@@ -147,11 +92,8 @@ k_batch_persistent(const BatchProblem<T>* __restrict__ probs, const BatchTask* _
   __shared__ long long s_item;
   __shared__ int s_task;
   __shared__ double red[32];
-  __shared__ float redf[2][32];  // warp partials of the compile-time x items, alternating
-  int par = 0;
   int* done = reinterpret_cast<int*>(queue + 1);
   int cur = 0;         // thread 0: the task of this block's previous item (items only increase)
-  int ct_loaded = 0;   // edge whose compile-time twiddle table this block's shared memory holds
   for (;;) {
     if (threadIdx.x == 0) {
       int task = -1;
@@ -189,12 +131,7 @@ k_batch_persistent(const BatchProblem<T>* __restrict__ probs, const BatchTask* _
     const BatchProblem<T>& P = probs[tk.prob];
     const long long local = s_item - tk.first;
     const Geo& g = P.g;
-    if ((tk.kind == kTaskFwd || tk.kind == kTaskX) && P.ct_n > 0 &&
-        ct_item(P, tk.kind, tk.a0, local, smem_raw, redf, par, ct_loaded == P.ct_n)) {
-      if (tk.kind == kTaskX) par ^= 1;
-      ct_loaded = P.ct_n;
-    } else if (tk.kind == kTaskFwd) {
-      ct_loaded = 0;  // the items below reuse the shared memory that held a twiddle table
+    if (tk.kind == kTaskFwd) {
       C* buf = reinterpret_cast<C*>(smem_raw);
       C* tw2 = buf + g.n2 * g.S;
       C* tw3 = tw2 + g.n2;
@@ -202,7 +139,6 @@ k_batch_persistent(const BatchProblem<T>* __restrict__ probs, const BatchTask* _
       for (int i = threadIdx.x; i < g.n3; i += blockDim.x) tw3[i] = P.tw3[i];
       fwd_yz_item(g, P.orb, P.couples, tk.a0, P.W, tw2, tw3, buf, local);
     } else if (tk.kind == kTaskX) {
-      ct_loaded = 0;
       C* buf = reinterpret_cast<C*>(smem_raw);
       C* tw1 = buf + g.n1 * g.S;
       C* tw3 = tw1 + g.n1;
@@ -210,7 +146,6 @@ k_batch_persistent(const BatchProblem<T>* __restrict__ probs, const BatchTask* _
       for (int i = threadIdx.x; i < g.n3; i += blockDim.x) tw3[i] = P.tw3[i];
       x_coulomb_item(g, P.couples, tk.a0, P.W, P.vtab, tw1, tw3, P.epart, P.energy_only != 0, buf, red, local);
     } else if (tk.kind == kTaskAcc) {
-      ct_loaded = 0;
       constexpr int ZC = ZChunk<T>::value;
       const int nzc = (g.n3 + ZC - 1) / ZC;
       const int zi = int(local % nzc);
@@ -237,7 +172,6 @@ k_batch_persistent(const BatchProblem<T>* __restrict__ probs, const BatchTask* _
         d[1] = hi;
       }
     } else {  // energy: E_x = scale * sum_g w_g sum_y epart[g][y], in a fixed order
-      ct_loaded = 0;  // (block_sum below uses only static shared memory; kept simple)
       double sacc = 0.0;
       for (int c = threadIdx.x; c < P.total_couples; c += blockDim.x) {
         const int4 cp = P.couples[c];

@@ -15,10 +15,10 @@ namespace ct {
 template <int N> struct Plan { static constexpr StagePlan p = stage_plan(N); };
 
 // element strides of x and y in a couple's transform W: [y][x][z] where the plane passes of
-// hfx_ct_plane.cuh run (edges that are a multiple of 8), else [x][y][z]
+// hfx_ct_plane.cuh run (edges that are a multiple of 4), else [x][y][z]
 template <int N> struct WStride {
-  static constexpr int x = N % 8 == 0 ? N : N * N;
-  static constexpr int y = N % 8 == 0 ? N * N : N;
+  static constexpr int x = N % 4 == 0 ? N : N * N;
+  static constexpr int y = N % 4 == 0 ? N * N : N;
 };
 
 // one in-place stage over LINES lines (element e of line l at buf[l*LS + e*ES])

@@ -11,7 +11,7 @@ namespace {
 constexpr int kN = HFX_CT_N;
 constexpr int kB = 8;
 // the forward and x passes of this edge: the plane passes of hfx_ct_plane.cuh where they exist
-template <int N, bool PLANE = N % 8 == 0> struct PlanePasses;
+template <int N, bool PLANE = N % 4 == 0> struct PlanePasses;
 template <int N> struct PlanePasses<N, true> {
   using G = ct::PlaneGeo<N>;
   using K = ct::PlaneCfg<N>;

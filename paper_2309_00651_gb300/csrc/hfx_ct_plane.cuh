@@ -1,4 +1,4 @@
-// Forward and x/Coulomb passes of the compile-time FP32 geometry for edges that are a multiple of 8.
+// Forward and x/Coulomb passes of the compile-time FP32 geometry for edges that are a multiple of 4.
 //
 // What bounds them: every point of a plane goes through shared memory once per exchange between
 // butterflies, and shared-memory throughput and issue slots (not HBM) set these passes' time.  So the
@@ -32,17 +32,21 @@ namespace hfx {
 namespace ct {
 
 template <int N> struct PlaneGeo {
-  static_assert(N % 8 == 0, "plane passes need an edge that is a multiple of 8");
+  static_assert(N % 4 == 0, "plane passes need an edge that is a multiple of 4");
   static constexpr int R = N / 4;                                   // large radix of z and x
-  static constexpr int E = R <= 12 ? 12 : (R - 5) / 8 * 8 + 12;     // >= R, 4 mod 8
+  static constexpr int E = (R + 3) / 8 * 8 + 4;                     // >= R, 4 mod 8
   static constexpr int SF = 4 * E + 3;                              // forward row stride
   static constexpr int SX = N + 2;                                  // x-pass row stride
   static constexpr StagePlan Y = stage_plan(N);
   static_assert(Y.ns == 2, "two y stages");
   static constexpr int RY0 = Y.r[0], RY1 = Y.r[1];
-  static constexpr int TW = 4 * R;                                  // z and x twiddles, then y's
+  static constexpr int TW = 4 * (R + R % 2);                        // z and x twiddles, then y's
   static constexpr int TWY = RY1 * RY0;
   static_assert(E >= R && E % 8 == 4, "bank-spreading stride of the z digits");
+  // place of output k of the large radix among its R: as two radices the runtime-geometry kernels know
+  // (plane_radices) would leave it, so that the tables and the pencil and batch kernels share the order
+  static constexpr PlaneRadices P = plane_radices(R);
+  static __host__ __device__ constexpr int place(int k) { return (k % P.a) * P.b + k / P.a; }
   static constexpr int smem_fwd = (N * SF + TW + TWY) * 8;
   static constexpr int smem_x = (N * SX + 2 + TW) * 8;
 };
@@ -55,27 +59,38 @@ template <int N> struct PlaneGeo {
 // a second buffer while one is transformed lost (399-425 us against 375): it halves the planes in work.
 template <int N> struct PlaneCfg;
 template <> struct PlaneCfg<32>  { static constexpr int fnt = 64,  fmb = 12, un = 4, xnt = 64,  xmb = 12; };
+template <> struct PlaneCfg<36>  { static constexpr int fnt = 96,  fmb = 8,  un = 2, xnt = 96,  xmb = 9; };
+template <> struct PlaneCfg<40>  { static constexpr int fnt = 96,  fmb = 8,  un = 2, xnt = 96,  xmb = 9; };
 template <> struct PlaneCfg<48>  { static constexpr int fnt = 96,  fmb = 8,  un = 2, xnt = 96,  xmb = 9; };
+template <> struct PlaneCfg<60>  { static constexpr int fnt = 128, fmb = 5,  un = 4, xnt = 128, xmb = 6; };
 template <> struct PlaneCfg<64>  { static constexpr int fnt = 128, fmb = 5,  un = 4, xnt = 128, xmb = 6; };
 template <> struct PlaneCfg<72>  { static constexpr int fnt = 160, fmb = 4,  un = 3, xnt = 128, xmb = 5; };
 template <> struct PlaneCfg<80>  { static constexpr int fnt = 160, fmb = 4,  un = 4, xnt = 160, xmb = 4; };
 template <> struct PlaneCfg<96>  { static constexpr int fnt = 192, fmb = 2,  un = 6, xnt = 384, xmb = 2; };
+template <> struct PlaneCfg<100> { static constexpr int fnt = 224, fmb = 2,  un = 4, xnt = 256, xmb = 2; };
+template <> struct PlaneCfg<108> { static constexpr int fnt = 224, fmb = 2,  un = 4, xnt = 256, xmb = 2; };
+template <> struct PlaneCfg<120> { static constexpr int fnt = 480, fmb = 1,  un = 4, xnt = 480, xmb = 1; };
 template <> struct PlaneCfg<128> { static constexpr int fnt = 512, fmb = 1,  un = 4, xnt = 512, xmb = 1; };
 
 // v[k] *= w^{e k} (or its conjugate); the table holds two consecutive k of one e in 16 bytes
 template <int R, bool CONJ>
-__device__ __forceinline__ void twiddle_zx(float2 (&v)[R], const float2* tw, int e) {
+__device__ __forceinline__ void twiddle_zx(cpair (&v)[R], const cpair* tw, int e) {
   const float4* t = reinterpret_cast<const float4*>(tw) + e;
 #pragma unroll
   for (int k = 0; k < R; k += 2) {
     const float4 w = t[(k / 2) * 4];
-    if (k > 0) v[k] = CONJ ? cmulc(v[k], make_float2(w.x, w.y)) : cmul(v[k], make_float2(w.x, w.y));
-    v[k + 1] = CONJ ? cmulc(v[k + 1], make_float2(w.z, w.w)) : cmul(v[k + 1], make_float2(w.z, w.w));
+    if (k > 0) v[k] = CONJ ? cmulc(v[k], cpair{w.x, w.y}) : cmul(v[k], cpair{w.x, w.y});
+    if (k + 1 < R) v[k + 1] = CONJ ? cmulc(v[k + 1], cpair{w.z, w.w}) : cmul(v[k + 1], cpair{w.z, w.w});
   }
 }
 
+__device__ __forceinline__ cpair ld_cg(const cpair* p) {
+  const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
+  return cpair{v.x, v.y};
+}
+
 // four consecutive complex values (32 bytes, 32-byte aligned) to global memory in one store
-__device__ __forceinline__ void st_c4(float2* p, float2 a, float2 b, float2 c, float2 d) {
+__device__ __forceinline__ void st_c4(float2* p, cpair a, cpair b, cpair c, cpair d) {
   asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(a.x), "f"(a.y), "f"(b.x),
                "f"(b.y), "f"(c.x), "f"(c.y), "f"(d.x), "f"(d.y)
                : "memory");
@@ -88,7 +103,7 @@ __device__ __forceinline__ void st_c4(float2* p, float2 a, float2 b, float2 c, f
 // ends the previous item's use of buf, so that their latency runs beside it.
 template <int N, int NT, int UN>
 __device__ __forceinline__ void product_to_smem(const float* __restrict__ orb, long long Ntot, int4 cp, int x,
-                                                float2* __restrict__ buf) {
+                                                cpair* __restrict__ buf) {
   using G = PlaneGeo<N>;
   constexpr int NV = N * G::R;
   const bool hasa = cp.x >= 0, hasb = cp.z >= 0;
@@ -131,11 +146,11 @@ __device__ __forceinline__ void product_to_smem(const float* __restrict__ orb, l
       const int i = i0 + u * NT;
       if ((NV % (UN * NT) == 0) || i < NV) {
         const int y = i / G::R, D = i - y * G::R;  // z = 4 D .. 4 D + 3
-        float2* d = buf + y * G::SF + D;
-        d[0] = make_float2(p[u].x * q[u].x, s[u].x);
-        d[G::E] = make_float2(p[u].y * q[u].y, s[u].y);
-        d[2 * G::E] = make_float2(p[u].z * q[u].z, s[u].z);
-        d[3 * G::E] = make_float2(p[u].w * q[u].w, s[u].w);
+        cpair* d = buf + y * G::SF + D;
+        d[0] = cpair{p[u].x * q[u].x, s[u].x};
+        d[G::E] = cpair{p[u].y * q[u].y, s[u].y};
+        d[2 * G::E] = cpair{p[u].z * q[u].z, s[u].z};
+        d[3 * G::E] = cpair{p[u].w * q[u].w, s[u].w};
       }
     }
   }
@@ -143,7 +158,7 @@ __device__ __forceinline__ void product_to_smem(const float* __restrict__ orb, l
 
 template <int N, int NT, int UN>
 __device__ __forceinline__ void fwd_plane_item(const float* __restrict__ orb, long long Ntot, int4 cp,
-                                               float2* __restrict__ W, float2* buf, const float2* tw, int cl, int x) {
+                                               float2* __restrict__ W, cpair* buf, const cpair* tw, int cl, int x) {
   using G = PlaneGeo<N>;
   constexpr int R = G::R, E = G::E, S = G::SF, PLANE = N * N, RY0 = G::RY0, RY1 = G::RY1;
   product_to_smem<N, NT, UN>(orb, Ntot, cp, x, buf);
@@ -152,26 +167,26 @@ __device__ __forceinline__ void fwd_plane_item(const float* __restrict__ orb, lo
 #pragma unroll 1
   for (int id = threadIdx.x; id < 4 * N; id += NT) {
     const int e = (id >> 2) & 3, y = (id >> 4) * 4 + (id & 3);
-    float2* p = buf + y * S + e * E;
-    float2 v[R];
+    cpair* p = buf + y * S + e * E;
+    cpair v[R];
 #pragma unroll
     for (int k = 0; k < R; ++k) v[k] = p[k];
-    Dft<R, -1, float2>::run(v);
+    Dft<R, -1, cpair>::run(v);
     twiddle_zx<R, false>(v, tw, e);
 #pragma unroll
-    for (int k = 0; k < R; ++k) p[k] = v[k];
+    for (int k = 0; k < R; ++k) p[G::place(k)] = v[k];
   }
   __syncthreads();
   // y: rows j + RY1 k of one column
 #pragma unroll 1
   for (int id = threadIdx.x; id < RY1 * N; id += NT) {
     const int j = id / N, c = id - j * N;
-    float2* p = buf + j * S + (c & 3) * E + (c >> 2);
-    float2 v[RY0];
+    cpair* p = buf + j * S + (c & 3) * E + (c >> 2);
+    cpair v[RY0];
 #pragma unroll
     for (int k = 0; k < RY0; ++k) v[k] = p[k * (RY1 * S)];
-    Dft<RY0, -1, float2>::run(v);
-    const float2* t = tw + G::TW + j * RY0;
+    Dft<RY0, -1, cpair>::run(v);
+    const cpair* t = tw + G::TW + j * RY0;
 #pragma unroll
     for (int k = 1; k < RY0; ++k) v[k] = cmul(v[k], t[k]);
 #pragma unroll
@@ -183,19 +198,19 @@ __device__ __forceinline__ void fwd_plane_item(const float* __restrict__ orb, lo
 #pragma unroll 1
   for (int id = threadIdx.x; id < R * RY0; id += NT) {
     const int Dy = id / R, D = id - Dy * R;
-    const float2* p = buf + Dy * (RY1 * S) + D;
-    float2 v[4][RY1];
+    const cpair* p = buf + Dy * (RY1 * S) + D;
+    cpair v[4][RY1];
 #pragma unroll
     for (int f = 0; f < RY1; ++f) {
-      float2 t[4];
+      cpair t[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) t[e] = p[f * S + e * E];
-      Dft<4, -1, float2>::run(t);
+      Dft<4, -1, cpair>::run(t);
 #pragma unroll
       for (int e = 0; e < 4; ++e) v[e][f] = t[e];
     }
 #pragma unroll
-    for (int e = 0; e < 4; ++e) Dft<RY1, -1, float2>::run(v[e]);
+    for (int e = 0; e < 4; ++e) Dft<RY1, -1, cpair>::run(v[e]);
     float2* d = w + Dy * (RY1 * PLANE) + 4 * D;
 #pragma unroll
     for (int f = 0; f < RY1; ++f) st_c4(d + f * PLANE, v[0][f], v[1][f], v[2][f], v[3][f]);
@@ -208,9 +223,9 @@ k_fwd_plane(const float* __restrict__ orb, long long Ntot, const int4* __restric
             float2* __restrict__ W, const float2* __restrict__ twg, int prefetch) {
   using G = PlaneGeo<N>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* tw = reinterpret_cast<float2*>(smem_raw);
-  float2* buf = tw + G::TW + G::TWY;
-  for (int i = threadIdx.x; i < G::TW + G::TWY; i += NT) tw[i] = twg[i];
+  cpair* tw = reinterpret_cast<cpair*>(smem_raw);
+  cpair* buf = tw + G::TW + G::TWY;
+  for (int i = threadIdx.x; i < G::TW + G::TWY; i += NT) tw[i] = cpair{twg[i].x, twg[i].y};
   const int ncl = c1 - c0, items = ncl * N;
   // x-major order: the blocks in flight work on the same x-plane of many couples, whose orbital planes
   // (the batch's orbitals at that x) are then read from DRAM once and from L2 after
@@ -245,8 +260,8 @@ k_fwd_plane(const float* __restrict__ orb, long long Ntot, const int4* __restric
 // red: [2][32] floats of shared memory used alternately (par) by consecutive items of a block
 template <int N, int NT>
 __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, const float* __restrict__ vtab,
-                                             double* __restrict__ epart, int energy_only, float2* buf,
-                                             const float2* tw, float (*red)[32], int par, int cl, int y) {
+                                             double* __restrict__ epart, int energy_only, cpair* buf,
+                                             const cpair* tw, float (*red)[32], int par, int cl, int y) {
   using G = PlaneGeo<N>;
   constexpr int R = G::R, S = G::SX, PLANE = N * N;
   float2* wc = W + ((long long)cl * N + y) * PLANE;
@@ -257,16 +272,16 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
 #pragma unroll 1
   for (int id = threadIdx.x; id < 4 * N; id += NT) {
     const int j = id / N, z = id - j * N;
-    const float2* src = wc + j * N + z;
-    float2* p = buf + j * S + z;
-    float2 v[R];
+    const cpair* src = reinterpret_cast<const cpair*>(wc) + j * N + z;
+    cpair* p = buf + j * S + z;
+    cpair v[R];
 #pragma unroll
-    for (int k = 0; k < R; ++k) v[k] = __ldcg(src + k * (4 * N));
-    Dft<R, -1, float2>::run(v);
+    for (int k = 0; k < R; ++k) v[k] = ld_cg(src + k * (4 * N));
+    Dft<R, -1, cpair>::run(v);
     twiddle_zx<R, false>(v, tw, j);
     if (NT <= 4 * N && id == threadIdx.x) __syncthreads();
 #pragma unroll
-    for (int k = 0; k < R; ++k) p[k * (4 * S) + 2 * ((k >> 1) & 1)] = v[k];
+    for (int k = 0; k < R; ++k) p[G::place(k) * (4 * S) + 2 * ((G::place(k) >> 1) & 1)] = v[k];
   }
   // the tile x = 4 X .. 4 X + 3, z = 4 Z .. 4 Z + 3: last forward x stage, v(G) and the energy, first
   // inverse x stage, first inverse z stage.  The plane's energy in FP32 (a few terms per thread, a tree
@@ -277,26 +292,28 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
 #pragma unroll 1
   for (int id = threadIdx.x; id < R * R; id += NT) {
     // lanes alternate between two x tiles whose rows are shifted against each other
-    const int q = id & 1, m = id >> 1, g = m / R, Z = m - g * R;
-    const int X = (R % 4 != 0 && g == R / 2 - 1) ? R - 2 + q : (g & 1) + 4 * (g >> 1) + 2 * q;
+    const int q = id & 1, m = R % 2 != 0 ? id : id >> 1, g = m / R, Z = m - g * R;
+    // (g of a pair of tiles two apart; what R leaves over: neighbours, or for odd R one by one)
+    constexpr int R4 = R / 4 * 4;
+    const int X = R % 2 != 0 ? id / R : (g >= R4 / 2 ? R4 + 2 * (g - R4 / 2) + q : (g & 1) + 4 * (g >> 1) + 2 * q);
     float4* p = reinterpret_cast<float4*>(buf + (4 * X) * S + 4 * Z + 2 * ((X >> 1) & 1));
     const float* vp = vy + (4 * X) * PLANE + 4 * Z;
     float4 vg4[4];
 #pragma unroll
     for (int f = 0; f < 4; ++f) vg4[f] = __ldg(reinterpret_cast<const float4*>(vp + f * PLANE));
-    float2 v[4][4];
+    cpair v[4][4];
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       const float4 a = p[f * (S / 2)], b = p[f * (S / 2) + 1];
-      v[0][f] = make_float2(a.x, a.y);
-      v[1][f] = make_float2(a.z, a.w);
-      v[2][f] = make_float2(b.x, b.y);
-      v[3][f] = make_float2(b.z, b.w);
+      v[0][f] = cpair{a.x, a.y};
+      v[1][f] = cpair{a.z, a.w};
+      v[2][f] = cpair{b.x, b.y};
+      v[3][f] = cpair{b.z, b.w};
     }
     float en = 0.f;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      Dft<4, -1, float2>::run(v[e]);
+      Dft<4, -1, cpair>::run(v[e]);
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
         const float vg = e == 0 ? vg4[f].x : e == 1 ? vg4[f].y : e == 2 ? vg4[f].z : vg4[f].w;
@@ -308,11 +325,11 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
     e_acc += en;
     if (!energy_only) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) Dft<4, 1, float2>::run(v[e]);
+      for (int e = 0; e < 4; ++e) Dft<4, 1, cpair>::run(v[e]);
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
-        float2 t[4] = {v[0][f], v[1][f], v[2][f], v[3][f]};
-        Dft<4, 1, float2>::run(t);
+        cpair t[4] = {v[0][f], v[1][f], v[2][f], v[3][f]};
+        Dft<4, 1, cpair>::run(t);
         p[f * (S / 2)] = make_float4(t[0].x, t[0].y, t[1].x, t[1].y);
         p[f * (S / 2) + 1] = make_float4(t[2].x, t[2].y, t[3].x, t[3].y);
       }
@@ -337,14 +354,15 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
   if (energy_only) return;
   // inverse z: elements e + 4 k of row x
 #pragma unroll 1
-  for (int id = threadIdx.x; id < 4 * N; id += NT) {
+  for (int id = threadIdx.x; id < (N + 7) / 8 * 32; id += NT) {
     const int e = (id >> 3) & 3, xg = id >> 5, x = xg * 8 + (id & 7);
-    float2* p = buf + x * S + 2 * (xg & 1) + e;
-    float2 v[R];
+    if (N % 8 != 0 && x >= N) continue;
+    cpair* p = buf + x * S + 2 * (xg & 1) + e;
+    cpair v[R];
 #pragma unroll
-    for (int k = 0; k < R; ++k) v[k] = p[4 * k];
+    for (int k = 0; k < R; ++k) v[k] = p[4 * G::place(k)];
     twiddle_zx<R, true>(v, tw, e);
-    Dft<R, 1, float2>::run(v);
+    Dft<R, 1, cpair>::run(v);
 #pragma unroll
     for (int k = 0; k < R; ++k) p[4 * k] = v[k];
   }
@@ -353,13 +371,13 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
 #pragma unroll 1
   for (int id = threadIdx.x; id < 4 * N; id += NT) {
     const int j = id / N, z = id - j * N;
-    const float2* p = buf + j * S + z;
-    float2 v[R];
+    const cpair* p = buf + j * S + z;
+    cpair v[R];
 #pragma unroll
-    for (int k = 0; k < R; ++k) v[k] = p[k * (4 * S) + 2 * ((k >> 1) & 1)];
+    for (int k = 0; k < R; ++k) v[k] = p[G::place(k) * (4 * S) + 2 * ((G::place(k) >> 1) & 1)];
     twiddle_zx<R, true>(v, tw, j);
-    Dft<R, 1, float2>::run(v);
-    float2* dst = wc + j * N + z;
+    Dft<R, 1, cpair>::run(v);
+    cpair* dst = reinterpret_cast<cpair*>(wc) + j * N + z;
 #pragma unroll
     for (int k = 0; k < R; ++k) dst[k * (4 * N)] = v[k];
   }
@@ -372,10 +390,10 @@ k_x_plane(const int4* __restrict__ couples, int c0, int c1, float2* __restrict__
   using G = PlaneGeo<N>;
   static_assert(NT % 32 == 0, "whole warps");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* tw = reinterpret_cast<float2*>(smem_raw);
-  float2* buf = tw + G::TW;
+  cpair* tw = reinterpret_cast<cpair*>(smem_raw);
+  cpair* buf = tw + G::TW;
   __shared__ float red[2][32];  // warp partials of the plane energy, double-buffered by item parity
-  for (int i = threadIdx.x; i < G::TW; i += NT) tw[i] = twg[i];
+  for (int i = threadIdx.x; i < G::TW; i += NT) tw[i] = cpair{twg[i].x, twg[i].y};
   int par = 0;
   const int items = (c1 - c0) * N;
   int it = blockIdx.x, cl = it / N;

@@ -100,7 +100,12 @@ void fwd_yz_tc(int n, int grid, cudaStream_t st, const float* orb, long long Nto
                int c1, float2* W, const unsigned char* dftb, int* err);
 }  // namespace dft
 
-#define HFX_CT_SIZES(X) X(32) X(48) X(64) X(72) X(80) X(90) X(96) X(128)
+// The cubic edges with passes of their own: the grids of water boxes between 36 and 128 that are even and
+// {2,3,5}-smooth.  Against the runtime-geometry passes, 48 orbitals, us a call: 36^3 1066 -> 426, 40^3 1328
+// -> 511, 50^3 2475 -> 1308, 54^3 2906 -> 1472, 60^3 3712 -> 1475, 100^3 20869 -> 8029, 108^3 26002 -> 9890,
+// 120^3 47380 -> 13677.  50, 54 and 90 (no multiple of 4: no 16-byte rows) run one stage at a time.
+#define HFX_CT_SIZES(X) \
+  X(32) X(36) X(40) X(48) X(50) X(54) X(60) X(64) X(72) X(80) X(90) X(96) X(100) X(108) X(120) X(128)
 #define HFX_CT_DECLARE(NN) const CtFns* ct_fns_##NN();
 HFX_CT_SIZES(HFX_CT_DECLARE)
 #undef HFX_CT_DECLARE
