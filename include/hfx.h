@@ -176,8 +176,8 @@ typedef struct {
  *   Rules: same argument rules per problem as hfx_apply; one distinct context per problem; every
  *   context needs the same precision and device and planes that fit in shared memory
  *   (HFX_ERR_UNSUPPORTED_GRID otherwise); each context's workspace must hold hfx_workspace_bytes
- *   for its problem; batched calls led by one context must not overlap on the GPU.  The persistent form's
- *   queue tables live in a device buffer owned by the first context (ctxs[0]); the first call that needs a larger one
+ *   for its problem; batched calls led by one context must not overlap on the GPU.  The queue tables
+ *   (sized by either form) live in a device buffer owned by the first context (ctxs[0]); the first call that needs a larger one
  *   allocates it (and synchronises the stream), so make that call before any stream capture --
  *   during capture such a call is rejected with HFX_ERR_INVALID_ARG.  Stops at the first problem
  *   whose arguments are rejected and returns that error. */

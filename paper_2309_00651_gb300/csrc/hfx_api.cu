@@ -1325,6 +1325,34 @@ extern "C" hfx_status hfx_apply_sequential(hfx_ctx* const* ctxs, const hfx_apply
   return HFX_OK;
 }
 
+// device tables of the persistent launch: queue header and done counters, tasks, problems
+struct BatchTables { size_t queue, tasks, probs, total; };
+template <typename T>
+static BatchTables batch_tables(size_t ntasks, size_t nprobs) {
+  BatchTables t;
+  size_t off = 0;
+  auto take = [&](size_t bytes) { size_t o = off; off += align256(bytes); return o; };
+  t.queue = take(sizeof(BatchQueue) + ntasks * sizeof(int));
+  t.tasks = take(ntasks * sizeof(BatchTask));
+  t.probs = take(nprobs * sizeof(BatchProblem<T>));
+  t.total = off;
+  return t;
+}
+static hfx_status ensure_batch_tables(hfx_ctx* lead, size_t bytes, cudaStream_t st) {
+  if (lead->batch_bytes >= bytes) return HFX_OK;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  HFX_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
+  if (cs != cudaStreamCaptureStatusNone)
+    return fail(HFX_ERR_INVALID_ARG, "the first batched call of this size on its lead context must come before stream capture");
+  if (lead->d_batch) { HFX_CUDA_TRY(cudaStreamSynchronize(st)); dev_free(lead->d_batch); }
+  lead->d_batch = nullptr;
+  lead->batch_bytes = 0;
+  cudaError_t e = dev_alloc(&lead->d_batch, bytes);
+  if (e != cudaSuccess) return fail(HFX_ERR_OOM, "cudaMalloc(%zu) for the batch tables failed: %s", bytes, cudaGetErrorString(e));
+  lead->batch_bytes = bytes;
+  return HFX_OK;
+}
+
 // The batch as one persistent launch (hfx_batch.cuh): per problem the staging launches (V cleared,
 // pairs placed, FP32 copy), then one launch of k_batch_persistent over the tasks of all problems.
 template <typename T>
@@ -1453,23 +1481,11 @@ static hfx_status batched_persistent(hfx_ctx* const* ctxs, const hfx_apply_args*
   long long total = 0;
   for (auto& t : tasks) { t.first = total; total += t.items; }
   const int ntasks = (int)tasks.size();
-  // device tables: queue header and done counters, tasks, problems
-  size_t off = 0;
-  auto take = [&](size_t bytes) { size_t o = off; off += align256(bytes); return o; };
-  const size_t o_queue = take(sizeof(BatchQueue) + (size_t)ntasks * sizeof(int));
-  const size_t o_tasks = take((size_t)ntasks * sizeof(BatchTask));
-  const size_t o_probs = take(probs.size() * sizeof(BatchProblem<T>));
-  if (lead->batch_bytes < off) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    HFX_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
-    if (cs != cudaStreamCaptureStatusNone)
-      return fail(HFX_ERR_INVALID_ARG, "the first batched call of this size on its lead context must come before stream capture");
-    if (lead->d_batch) { HFX_CUDA_TRY(cudaStreamSynchronize(st)); dev_free(lead->d_batch); }
-    lead->d_batch = nullptr;
-    lead->batch_bytes = 0;
-    cudaError_t e = dev_alloc(&lead->d_batch, off);
-    if (e != cudaSuccess) return fail(HFX_ERR_OOM, "cudaMalloc(%zu) for the batch tables failed: %s", off, cudaGetErrorString(e));
-    lead->batch_bytes = off;
+  const BatchTables tb = batch_tables<T>(ntasks, probs.size());
+  const size_t o_queue = tb.queue, o_tasks = tb.tasks, o_probs = tb.probs;
+  {
+    const hfx_status sa = ensure_batch_tables(lead, tb.total, st);
+    if (sa != HFX_OK) return sa;
   }
   char* base = (char*)lead->d_batch;
   hfx_status s = put_table(base + o_tasks, tasks.data(), tasks.size() * sizeof(BatchTask), st);
@@ -1502,9 +1518,11 @@ static bool batch_is_small(hfx_ctx* const* ctxs, const hfx_apply_args* args, int
 
 // The batch as one evaluation per problem, each with its own passes on its context's second stream, forked
 // from the caller's stream and joined to it: launches of different problems fill each other's tails.
-// Everything that can be refused is refused before anything is enqueued.
+// Everything that can be refused is refused before anything is enqueued, and by the persistent form's rules
+// (its tables are sized too, so a batch of this size can be captured in either form from then on).
 static hfx_status batched_forked(hfx_ctx* const* ctxs, const hfx_apply_args* args, int32_t n, cudaStream_t st) {
   std::vector<Schedule*> scheds(n, nullptr);
+  size_t ntasks = 0, nprobs = 0;
   for (int32_t k = 0; k < n; ++k) {
     hfx_ctx* c = ctxs[k];
     if (c->pencil)
@@ -1518,6 +1536,14 @@ static hfx_status batched_forked(hfx_ctx* const* ctxs, const hfx_apply_args* arg
     const size_t need = layout_of(c, *scheds[k], args[k].n_orb, false).total;
     if (!c->ws || c->ws_bytes < need)
       return fail(HFX_ERR_OOM, "problem %d: workspace too small: have %zu bytes, need %zu", (int)k, c->ws_bytes, need);
+    const size_t acc = args[k].flags & HFX_ENERGY_ONLY ? 0 : 1;
+    ntasks += scheds[k]->nbatches * (2 + acc) + (c->prec == HFX_PREC_FP32 ? acc : 0) + 1;
+    ++nprobs;
+  }
+  if (nprobs > 0) {
+    const size_t bytes = (ctxs[0]->prec == HFX_PREC_FP64 ? batch_tables<double>(ntasks, nprobs) : batch_tables<float>(ntasks, nprobs)).total;
+    const hfx_status s = ensure_batch_tables(ctxs[0], bytes, st);
+    if (s != HFX_OK) return s;
   }
   hfx_status result = HFX_OK;
   HFX_CUDA_TRY(cudaEventRecord(ctxs[0]->ev_fork, st));
