@@ -773,7 +773,7 @@ static Layout layout_of(const hfx_ctx* c, const Schedule& S, int n_orb, bool sec
   // a second transform buffer when batches are pipelined on two streams
   L.W2 = take(second_buffer ? (size_t)S.max_batch_couples * c->N * cplx_size(c) : 0);
   L.epart = take((size_t)S.max_total_couples * eparts(c) * sizeof(double));
-  L.eblk = take((size_t)64 * sizeof(double));  // per-block energy sums (kEnergyBlocks)
+  L.eblk = take((size_t)64 * sizeof(double));  // per-block energy sums (kEnergyBlocks), the count of finished blocks
   L.couples = take(couple_table_bytes(S));
   L.total = off;
   return L;
@@ -781,8 +781,10 @@ static Layout layout_of(const hfx_ctx* c, const Schedule& S, int n_orb, bool sec
 
 extern "C" size_t hfx_workspace_bytes(const hfx_ctx* c, int32_t n_orb, int64_t n_pairs) {
   if (!c || n_orb <= 0 || n_pairs < 0) return 0;
-  Schedule S = make_host_schedule(c, n_orb);
   (void)n_pairs;
+  const auto it = c->sched.find(n_orb);  // (dropped when a setting that it depends on changes)
+  if (it != c->sched.end()) return layout_of(c, *it->second, n_orb, two_buffers(c, *it->second)).total;
+  const Schedule S = make_host_schedule(c, n_orb);
   return layout_of(c, S, n_orb, two_buffers(c, S)).total;
 }
 
@@ -819,25 +821,29 @@ static hfx_status get_schedule(hfx_ctx* c, int n_orb, Schedule** out) {
 // ------------------------------------------------------------------------------------
 // pair-list staging kernels (validate, bucket by block pair and weight class, stable order)
 // ------------------------------------------------------------------------------------
-__global__ void k_cast_f32(const double* __restrict__ src, float* __restrict__ dst, long long n) {
-  const long long n2 = n / 2;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n2; i += (long long)gridDim.x * blockDim.x) {
-    const double2 v = reinterpret_cast<const double2*>(src)[i];
-    reinterpret_cast<float2*>(dst)[i] = make_float2((float)v.x, (float)v.y);
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0 && (n & 1)) dst[n - 1] = (float)src[n - 1];
-}
-
 // every listed pair goes to its fixed place in the canonical couple layout of its block pair;
 // entries outside 0 <= i <= j < n_orb, and second copies of a pair, are flagged and skipped.
 // dead_words (the TMA dense pass: slots of at most 32 couples) loses the bit of every couple that gets
 // a pair, and off-diagonal pairs with the last, ragged block are laid out with its orbitals as rows
-__global__ void k_plan_place(const int2* __restrict__ pairs, long long P, int n_orb, int bsize, int nb,
-                             const int* __restrict__ slot_of_bp, const int* __restrict__ slot_couple_base,
-                             int4* __restrict__ couples, unsigned* __restrict__ dead_words,
-                             int* __restrict__ err) {
-  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x) {
-    const int2 ij = pairs[p];
+struct PlaceArgs {
+  const int2* pairs;
+  long long P;
+  int n_orb, bsize, nb;
+  const int* slot_of_bp;
+  const int* slot_couple_base;
+  int4* couples;
+  unsigned* dead_words;
+  int* err;
+};
+__device__ __forceinline__ void place_pairs(const PlaceArgs& A, long long first, long long step) {
+  const int n_orb = A.n_orb, bsize = A.bsize, nb = A.nb;
+  const int* __restrict__ slot_of_bp = A.slot_of_bp;
+  const int* __restrict__ slot_couple_base = A.slot_couple_base;
+  int4* couples = A.couples;
+  unsigned* dead_words = A.dead_words;
+  int* err = A.err;
+  for (long long p = first; p < A.P; p += step) {
+    const int2 ij = A.pairs[p];
     const int i = ij.x, j = ij.y;
     if (!(i >= 0 && j < n_orb && i <= j)) { atomicOr(err, kErrBadPair); continue; }
     const int bi = i / bsize, bj = j / bsize;
@@ -864,41 +870,106 @@ __global__ void k_plan_place(const int2* __restrict__ pairs, long long P, int n_
   }
 }
 
-// E_x = scale * sum_g w_g sum_y epart[g][y], in two deterministic launches: block b of
-// k_energy_blocks sums couples [b*chunk, (b+1)*chunk) in a fixed order, k_energy_final sums the
-// kEnergyBlocks block results in order and stores or accumulates E_x
-constexpr int kEnergyBlocks = 64;
+__global__ void k_plan_place(const PlaceArgs A) {
+  place_pairs(A, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
+}
 
-__global__ void __launch_bounds__(256) k_energy_blocks(const double* __restrict__ epart, const int4* __restrict__ couples,
-                                                       int total, int n2, double* __restrict__ eblk) {
+// The first launch of a call: what has to start as zero (the V_x phi accumulator, 16-byte words) is
+// cleared, the FP64 orbitals are rounded to the passes' FP32 copy (src == NULL: not needed), the couple
+// table starts as all ones and the energy sum's count of finished blocks as zero.  A short pair list is
+// also placed here, by the first block alone (`place`: its table needs no other block), which saves a
+// launch; one launch and the placement's were four, about 4 us of a small call.
+constexpr long long kPlaceHere = 1024;
+__global__ void __launch_bounds__(256) k_stage(uint4* __restrict__ zero, long long nzero, const double* __restrict__ src,
+                                               float* __restrict__ dst, long long n, int* __restrict__ table,
+                                               int table_words, unsigned* __restrict__ count, int place,
+                                               const PlaceArgs A) {
+  long long first = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+  if (first == 0) *count = 0u;
+  if (place) {
+    if (blockIdx.x == 0) {
+      for (int i = threadIdx.x; i < table_words; i += blockDim.x) table[i] = -1;
+      __threadfence();
+      __syncthreads();
+      place_pairs(A, threadIdx.x, blockDim.x);
+      return;
+    }
+    first -= blockDim.x;
+    step -= blockDim.x;
+  } else {
+    for (long long i = first; i < table_words; i += step) table[i] = -1;
+  }
+  for (long long i = first; i < nzero; i += step) zero[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (src)
+    for (long long i = first; i < n / 4; i += step) {  // (three even edges: n is a multiple of 8)
+      const double2 u = __ldcs(reinterpret_cast<const double2*>(src) + 2 * i);
+      const double2 v = __ldcs(reinterpret_cast<const double2*>(src) + 2 * i + 1);
+      reinterpret_cast<float4*>(dst)[i] = make_float4((float)u.x, (float)u.y, (float)v.x, (float)v.y);
+    }
+}
+
+// E_x = scale * sum_g w_g sum_y epart[g][y] by the first `ne` blocks of the call's last launch: block b
+// sums couples [b*chunk, (b+1)*chunk) in a fixed order, and the block that finishes last adds the ne block
+// results in order and stores or accumulates E_x (deterministic: who is last does not change the sum).
+// The other blocks widen V_x phi (FP32 path): V_x phi (FP64) = (accumulate ? V_x phi : 0) + the call's FP32
+// accumulator, exactly and with integer operations (FP32 subnormals flush to zero); n is a multiple of 4
+constexpr int kEnergyBlocks = 63;
+
+__device__ __forceinline__ void widen_v4(const float* __restrict__ v32, double* __restrict__ v, long long i4,
+                                         int accumulate) {
+  const float4 a = __ldcs(reinterpret_cast<const float4*>(v32) + i4);
+  double2 lo = make_double2(ct::widen_exact(a.x), ct::widen_exact(a.y));
+  double2 hi = make_double2(ct::widen_exact(a.z), ct::widen_exact(a.w));
+  double2* d = reinterpret_cast<double2*>(v) + 2 * i4;
+  if (accumulate) {
+    const double2 o0 = d[0], o1 = d[1];
+    lo.x += o0.x; lo.y += o0.y; hi.x += o1.x; hi.y += o1.y;
+  }
+  d[0] = lo;
+  d[1] = hi;
+}
+
+__global__ void __launch_bounds__(256) k_finish(const double* __restrict__ epart, const int4* __restrict__ couples,
+                                                int total, int n2, double* __restrict__ eblk,
+                                                unsigned* __restrict__ count, int ne, double scale, int accumulate,
+                                                double* __restrict__ ex, const float* __restrict__ v32,
+                                                double* __restrict__ v, long long n) {
+  if ((int)blockIdx.x >= ne) {
+    for (long long i = (blockIdx.x - ne) * (long long)blockDim.x + threadIdx.x; i < n / 4;
+         i += (long long)(gridDim.x - ne) * blockDim.x)
+      widen_v4(v32, v, i, accumulate);
+    return;
+  }
   __shared__ double red[32];
-  const int chunk = (total + gridDim.x - 1) / gridDim.x;
+  __shared__ int last;
+  const int chunk = (total + ne - 1) / ne;
   const int g0 = blockIdx.x * chunk, g1 = min(total, g0 + chunk);
   double s = 0.0;
-  for (int g = g0 + threadIdx.x; g < g1; g += blockDim.x) {
+  for (int i = threadIdx.x; i < (g1 - g0) * n2; i += blockDim.x) {
+    const int g = g0 + i / n2;
     const int4 cp = couples[g];
     if (couple_empty(cp)) continue;
     // both halves of a couple share a weight class: diagonal pairs count once, others twice
     const bool diag = cp.x >= 0 ? cp.x == cp.y : cp.z == cp.w;
-    double t = 0.0;
-    for (int y = 0; y < n2; ++y) t += epart[(long long)g * n2 + y];
-    s += (diag ? 1.0 : 2.0) * t;
+    const double t = epart[(long long)g0 * n2 + i];
+    s += diag ? t : 2.0 * t;
   }
   const double tot = block_sum(s, red);
-  if (threadIdx.x == 0) eblk[blockIdx.x] = tot;
-}
-
-__global__ void k_energy_final(const double* __restrict__ eblk, int nb, double scale, int accumulate,
-                               double* __restrict__ ex) {
-  double t = 0.0;
-  for (int b = 0; b < nb; ++b) t += eblk[b];
-  ex[0] = (accumulate ? ex[0] : 0.0) + scale * t;
-}
-
-static void launch_energy(const double* epart, const int4* couples, int total, int n2, double* eblk, double scale,
-                          bool accumulate, double* ex, cudaStream_t st) {
-  k_energy_blocks<<<kEnergyBlocks, 256, 0, st>>>(epart, couples, total, n2, eblk);
-  k_energy_final<<<1, 1, 0, st>>>(eblk, kEnergyBlocks, scale, accumulate ? 1 : 0, ex);
+  if (threadIdx.x == 0) {
+    eblk[blockIdx.x] = tot;
+    __threadfence();
+    last = atomicAdd(count, 1u) == (unsigned)ne - 1u;
+  }
+  __syncthreads();
+  if (!last) return;
+  if (threadIdx.x < 32) {
+    __threadfence();
+    double t = threadIdx.x < ne ? __ldcg(eblk + threadIdx.x) : 0.0;
+    if (threadIdx.x + 32 < ne) t += __ldcg(eblk + threadIdx.x + 32);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (threadIdx.x == 0) ex[0] = (accumulate ? ex[0] : 0.0) + scale * t;
+  }
 }
 
 __global__ void k_set_scalar(double* p, double v) { *p = v; }
@@ -961,26 +1032,6 @@ static GuardSet guard_set(const Layout& L) {
   g.n = L.nguard;
   for (int k = 0; k < 8; ++k) g.off[k] = L.guard[k];
   return g;
-}
-
-// V_x phi (FP64) = (accumulate ? V_x phi : 0) + the call's FP32 accumulator, widened exactly with
-// integer operations (FP32 subnormals flush to zero); n is a multiple of 4
-__device__ __forceinline__ void widen_v4(const float* __restrict__ v32, double* __restrict__ v, long long i4,
-                                         int accumulate) {
-  const float4 a = __ldcs(reinterpret_cast<const float4*>(v32) + i4);
-  double2 lo = make_double2(ct::widen_exact(a.x), ct::widen_exact(a.y));
-  double2 hi = make_double2(ct::widen_exact(a.z), ct::widen_exact(a.w));
-  double2* d = reinterpret_cast<double2*>(v) + 2 * i4;
-  if (accumulate) {
-    const double2 o0 = d[0], o1 = d[1];
-    lo.x += o0.x; lo.y += o0.y; hi.x += o1.x; hi.y += o1.y;
-  }
-  d[0] = lo;
-  d[1] = hi;
-}
-__global__ void k_widen_v(const float* __restrict__ v32, double* __restrict__ v, long long n, int accumulate) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n / 4; i += (long long)gridDim.x * blockDim.x)
-    widen_v4(v32, v, i, accumulate);
 }
 
 // Small tables reach device memory as kernel arguments (8 KiB per launch): no host buffer has to
@@ -1152,12 +1203,6 @@ static hfx_status run_passes(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
     }
     if (pipe) HFX_CUDA_TRY(cudaEventRecord(c->ev_p3[b & 1], st));
   }
-  if (std::is_same<T, float>::value && !energy_only) {
-    const long long n = (long long)n_orb * g.N;
-    const int blocks = (int)std::min<long long>((n / 4 + 255) / 256, (long long)c->sm_count * 16);
-    k_widen_v<<<std::max(blocks, 1), 256, 0, st>>>((const float*)vacc, vxphi, n, (flags & HFX_ACCUMULATE) ? 1 : 0);
-    HFX_CUDA_TRY(cudaGetLastError());
-  }
   return HFX_OK;
 }
 
@@ -1199,33 +1244,32 @@ static hfx_status stage_call(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
   char* ws = env.ws;
   const bool accumulate = (flags & HFX_ACCUMULATE) != 0;
   const bool energy_only = (flags & HFX_ENERGY_ONLY) != 0;
-  if (c->prec == HFX_PREC_FP32) {
-    // the FP32 accumulator starts at zero; V_x phi itself is written (or added to) at the end
-    if (!energy_only) HFX_CUDA_TRY(cudaMemsetAsync(ws + L.v32, 0, (size_t)n_orb * c->N * sizeof(float), st));
-  } else if (!accumulate && !energy_only) {
-    HFX_CUDA_TRY(cudaMemsetAsync(vxphi, 0, (size_t)n_orb * c->N * sizeof(double), st));
-  }
+  // the FP32 accumulator starts at zero (V_x phi itself is written, or added to, at the end); on the FP64
+  // path V_x phi does, unless the call accumulates
+  void* zero = nullptr;
+  long long zero_bytes = 0;
+  const long long n = (long long)n_orb * c->N;
+  if (c->prec == HFX_PREC_FP32 && !energy_only) { zero = ws + L.v32; zero_bytes = n * 4; }
+  if (c->prec == HFX_PREC_FP64 && !accumulate && !energy_only) { zero = vxphi; zero_bytes = n * 8; }
+  const bool cast = c->prec == HFX_PREC_FP32 && !(flags & HFX_ORBITALS_F32);
+  float* dst = (float*)(ws + L.orb32);
   int4* couples = (int4*)(ws + L.couples);
-  HFX_CUDA_TRY(cudaMemsetAsync(couples, 0xff, couple_table_bytes(S), st));
-  {
-    const int threads = 256;
-    const int blocks = (int)std::max<long long>(1, std::min<long long>((n_pairs + threads - 1) / threads,
-                                                                        (long long)c->sm_count * 8));
-    k_plan_place<<<blocks, threads, 0, st>>>((const int2*)pairs, n_pairs, n_orb, S.b, S.nb, S.d_slot_of_bp,
-                                             S.d_slot_couple_base, couples,
-                                             S.ragged_rows ? (unsigned*)(couples + S.max_total_couples) : nullptr,
-                                             c->d_err);
-  }
+  const PlaceArgs A{(const int2*)pairs, n_pairs, n_orb, S.b, S.nb, S.d_slot_of_bp, S.d_slot_couple_base, couples,
+                    S.ragged_rows ? (unsigned*)(couples + S.max_total_couples) : nullptr, c->d_err};
+  const bool place = n_pairs <= kPlaceHere;
+  const int words = (int)(couple_table_bytes(S) / 4);
+  const long long work = std::max<long long>(std::max(zero_bytes / 16, cast ? n / 4 : 0), place ? 1 : words);
+  const int blocks = (int)std::min<long long>((work + 255) / 256, (long long)c->sm_count * 16) + (place ? 1 : 0);
+  k_stage<<<blocks, 256, 0, st>>>((uint4*)zero, zero_bytes / 16, cast ? (const double*)orbitals : nullptr, dst, n,
+                                  (int*)couples, words, (unsigned*)(ws + L.eblk + kEnergyBlocks * sizeof(double)),
+                                  place ? 1 : 0, A);
   HFX_CUDA_TRY(cudaGetLastError());
-  *orb_pass = orbitals;
-  if (c->prec == HFX_PREC_FP32 && !(flags & HFX_ORBITALS_F32)) {
-    float* dst = (float*)(ws + L.orb32);
-    const long long n = (long long)n_orb * c->N;
-    const int blocks = (int)std::min<long long>((n / 2 + 255) / 256 + 1, (long long)c->sm_count * 16);
-    k_cast_f32<<<blocks, 256, 0, st>>>((const double*)orbitals, dst, n);
+  if (!place) {
+    const int pb = (int)std::min<long long>((n_pairs + 255) / 256, (long long)c->sm_count * 8);
+    k_plan_place<<<pb, 256, 0, st>>>(A);
     HFX_CUDA_TRY(cudaGetLastError());
-    *orb_pass = dst;
   }
+  *orb_pass = cast ? (const void*)dst : orbitals;
   return HFX_OK;
 }
 
@@ -1245,7 +1289,7 @@ static hfx_status apply_with(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
   const void* orb = nullptr;
   hfx_status rs;
   {
-    NvtxRange r("hfx stage: V clear, pair placement, FP32 copy");
+    NvtxRange r("hfx stage: V clear, FP32 copy, pair placement");
     rs = stage_call(c, S, L, env, orbitals, n_orb, pairs, n_pairs, flags, vxphi, st, &orb);
   }
   if (rs != HFX_OK) return rs;
@@ -1261,9 +1305,17 @@ static hfx_status apply_with(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
   const double scale = -0.5 * c->alpha * c->omega / ((double)c->N * (double)c->N);
   cudaEvent_t e_en = env.prof ? prof_mark(c, st) : nullptr;
   {
-    NvtxRange r("hfx energy sum");
-    launch_energy((const double*)(ws + L.epart), (const int4*)(ws + L.couples), (int)S.max_total_couples, eparts(c),
-                  (double*)(ws + L.eblk), scale, accumulate, ex_dev, st);
+    NvtxRange r("hfx energy sum, V_x phi widened");
+    const int total = (int)S.max_total_couples, n2 = eparts(c);
+    // about 2048 partial sums a block
+    const int ne = (int)std::max<long long>(1, std::min<long long>({(long long)kEnergyBlocks, (long long)total,
+                                                                   (long long)total * n2 / 2048}));
+    const bool widen = c->prec == HFX_PREC_FP32 && !(flags & HFX_ENERGY_ONLY);
+    const long long n = (long long)n_orb * c->N;
+    const int wb = widen ? (int)std::max<long long>(1, std::min<long long>((n / 4 + 255) / 256, (long long)c->sm_count * 16)) : 0;
+    k_finish<<<ne + wb, 256, 0, st>>>((const double*)(ws + L.epart), (const int4*)(ws + L.couples), total, n2,
+                                      (double*)(ws + L.eblk), (unsigned*)(ws + L.eblk + kEnergyBlocks * sizeof(double)),
+                                      ne, scale, accumulate ? 1 : 0, ex_dev, (const float*)(ws + L.v32), vxphi, n);
   }
   if (env.prof) prof_close(c, kProfEnergy, e_en, st);
 #ifdef HFX_DEBUG
@@ -1632,13 +1684,11 @@ extern "C" hfx_status hfx_plan_stats(const hfx_ctx* c, int32_t n_orb, int64_t n_
   const bool eo = (flags & HFX_ENERGY_ONLY) != 0;
   long long launches = 0;
   if (n_pairs > 0) {
-    launches = 1 /* placement */ + 2 /* energy */ + (long long)S.nbatches * 2;
+    launches = 1 /* staging */ + (n_pairs > kPlaceHere) /* placement */ + 1 /* energy, widening */ + (long long)S.nbatches * 2;
     if (!eo)
       for (int b = 0; b < S.nbatches; ++b)
         launches += (S.dense_begin[b + 1] > S.dense_begin[b]) + (S.generic_begin[b + 1] > S.generic_begin[b]) +
                     (S.diag_begin[b + 1] > S.diag_begin[b]);
-    if (c->prec == HFX_PREC_FP32 && !(flags & HFX_ORBITALS_F32)) launches += 1; /* FP64 -> FP32 orbitals */
-    if (c->prec == HFX_PREC_FP32 && !eo) launches += 1;                         /* FP32 V accumulator -> V */
   } else if (!(flags & HFX_ACCUMULATE)) {
     launches = 1;
   }
