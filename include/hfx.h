@@ -249,7 +249,7 @@ hfx_status hfx_sync_status(hfx_ctx* c, void* cuda_stream);
  * not depend on them beyond rounding order):
  *   block       : orbitals per block (1..32, default 8; 4 and 8 have register-accumulating
  *                 kernels for full off-diagonal block pairs);
- *   batch_bytes : device memory for one batch of packed transforms (default 1 GiB);
+ *   batch_bytes : device memory for one batch of packed transforms (default 2 GiB);
  *   pipeline    : nonzero = the forward/x passes of the next batch run on a second stream beside
  *                 the accumulate pass of the current one (two transform buffers), 0 = one stream.
  * Synchronises the device when cached schedules have to be dropped; not during stream capture.

@@ -175,7 +175,10 @@ struct hfx_ctx {
   void* ws = nullptr;
   size_t ws_bytes = 0;
   int bsize = 8;
-  size_t transform_budget = size_t(1) << 30;
+  // bytes of transforms in one batch (of two buffers).  Larger launches have smaller tails: a call of 256
+  // orbitals on 96^3 took 150.3, 145.2, 137.6 and 135.5 ms with 0.5, 1, 2 and 4 GiB, 64 on 128^3 29.0, 27.4,
+  // 26.3 and 26.3; rounds that fit 1 GiB (72^3) do not change
+  size_t transform_budget = size_t(2) << 30;
   int blocks_fwd = 1, blocks_x = 1;
   int gen_grp = 1, gen_phi = 0;  // generic accumulate pass: couples per group, orbital tiles on chip
   // second stream and events: the forward and x passes of batch b+1 run beside the accumulate
@@ -737,15 +740,24 @@ extern "C" hfx_status hfx_set_workspace(hfx_ctx* c, void* dev_ptr, size_t bytes)
 
 static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
+// Batches share a launch of the forward and x passes up to kGroupMax bytes of transforms, where one of them
+// takes at least kGroupMin: smaller ones stay in L2 from pass to pass and overlap better on two streams.
+// Compile-time FP32 passes only (FP64, 48^3, 24 orbitals lost 4%).  Measured, us a call, apart / together:
+// 64^3 with 64 orbitals 2544 / 2419, 60^3 with 72 3039 / 2968, 72^3 with 32 1042 / 1008, 48^3 with 48 693 /
+// 666; together lost at 48^3 with 24 (201 / 221) and 32^3 with 64 (371 / 409), whose batches are 44 and 33 MB.
+constexpr size_t kGroupMin = size_t(64) << 20, kGroupMax = size_t(1) << 30;
+
 static Schedule make_host_schedule(const hfx_ctx* c, int n_orb) {
   Schedule S;
   build_schedule(S, n_orb, c->bsize, c->transform_budget, (size_t)c->N * cplx_size(c), dense_available(c),
                  diag_available(c), ragged_dense(c));
+  const size_t per = (size_t)c->N * cplx_size(c);
+  build_groups(S, c->ct && S.max_batch_couples * per >= kGroupMin ? (long long)(std::min(kGroupMax, c->transform_budget) / per) : 0);
   return S;
 }
 
 // two transform buffers when the batches of a call are pipelined on the context's two streams
-static bool two_buffers(const hfx_ctx* c, const Schedule& S) { return S.nbatches > 1 && c->side && c->pipeline; }
+static bool two_buffers(const hfx_ctx* c, const Schedule& S) { return S.ngroups > 1 && c->side && c->pipeline; }
 
 // the couple table, then for the TMA dense pass (slots of at most 32 couples) one word per slot whose set
 // bits are the couples without pairs; both start as all ones
@@ -769,9 +781,9 @@ static Layout layout_of(const hfx_ctx* c, const Schedule& S, int n_orb, bool sec
   L.orb32 = take(orb32_bytes);
   // FP32 path: the call's FP32 accumulator of V_x phi (widened into the caller's FP64 array once)
   L.v32 = take(c->prec == HFX_PREC_FP32 ? (size_t)n_orb * c->N * 4 : 0);
-  L.W = take((size_t)S.max_batch_couples * c->N * cplx_size(c));
+  L.W = take((size_t)S.max_group_couples * c->N * cplx_size(c));
   // a second transform buffer when batches are pipelined on two streams
-  L.W2 = take(second_buffer ? (size_t)S.max_batch_couples * c->N * cplx_size(c) : 0);
+  L.W2 = take(second_buffer ? (size_t)S.max_group_couples * c->N * cplx_size(c) : 0);
   L.epart = take((size_t)S.max_total_couples * eparts(c) * sizeof(double));
   L.eblk = take((size_t)64 * sizeof(double));  // per-block energy sums (kEnergyBlocks), the count of finished blocks
   L.couples = take(couple_table_bytes(S));
@@ -1077,7 +1089,7 @@ static hfx_status run_passes(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
                              uint32_t flags, double* vxphi, cudaStream_t st) {
   char* ws = env.ws;
   using C = cx<T>;
-  const bool pipe = S.nbatches > 1 && env.side != nullptr && c->pipeline;
+  const bool pipe = S.ngroups > 1 && env.side != nullptr && c->pipeline;
   // what the accumulate passes add into: V_x phi itself (FP64), or the call's FP32 accumulator
   T* vacc = std::is_same<T, float>::value ? (T*)(ws + L.v32) : (T*)vxphi;
   auto mark = [&](cudaStream_t s) { return env.prof ? prof_mark(c, s) : nullptr; };
@@ -1100,8 +1112,8 @@ static hfx_status run_passes(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
   if (std::is_same<T, float>::value && ragged_dense(c) && S.b == 8 && !energy_only) {
     const int cpi = dense_rows_ct(g.n1) * (S.b / 2);
     dense_tma =
-        encode_dense_maps(&tmW[0], Wbuf[0], S.max_batch_couples, cpi, g.wx, g.wy, &tmOrb, orb, &tmV, vacc, n_orb, g.n1) &&
-        encode_dense_maps(&tmW[1], Wbuf[1], S.max_batch_couples, cpi, g.wx, g.wy, &tmOrb, orb, &tmV, vacc, n_orb, g.n1);
+        encode_dense_maps(&tmW[0], Wbuf[0], S.max_group_couples, cpi, g.wx, g.wy, &tmOrb, orb, &tmV, vacc, n_orb, g.n1) &&
+        encode_dense_maps(&tmW[1], Wbuf[1], S.max_group_couples, cpi, g.wx, g.wy, &tmOrb, orb, &tmV, vacc, n_orb, g.n1);
     // the buffers are 16-byte aligned and the edges multiples of 4, so the driver has no reason to refuse
     if (!dense_tma) return fail(HFX_ERR_CUDA, "cuTensorMapEncodeTiled refused the dense pass's tensor maps");
   }
@@ -1111,11 +1123,11 @@ static hfx_status run_passes(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
     HFX_CUDA_TRY(cudaEventRecord(c->ev_fork, st));
     HFX_CUDA_TRY(cudaStreamWaitEvent(fs, c->ev_fork, 0));
   }
-  for (int b = 0; b < S.nbatches; ++b) {
-    C* W = Wbuf[b & 1];
-    // buffer b & 1 was last read by the accumulate pass of batch b - 2
-    if (pipe && b >= 2) HFX_CUDA_TRY(cudaStreamWaitEvent(fs, c->ev_p3[b & 1], 0));
-    const int s0 = S.batch_slot_begin[b], s1 = S.batch_slot_begin[b + 1];
+  for (int q = 0; q < S.ngroups; ++q) {
+    C* W = Wbuf[q & 1];
+    // buffer q & 1 was last read by the accumulate passes of group q - 2
+    if (pipe && q >= 2) HFX_CUDA_TRY(cudaStreamWaitEvent(fs, c->ev_p3[q & 1], 0));
+    const int s0 = S.batch_slot_begin[S.group_begin[q]], s1 = S.batch_slot_begin[S.group_begin[q + 1]];
     const int c0 = S.slot_couple_base[s0], c1 = S.slot_couple_base[s1];
     const long long items1 = (long long)(c1 - c0) * g.n1, items2 = (long long)(c1 - c0) * g.n2;
     const int grid1 = (int)std::min<long long>(items1, (long long)c->sm_count * c->blocks_fwd * 8);
@@ -1167,12 +1179,12 @@ static hfx_status run_passes(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
       HFX_CUDA_TRY(cudaEventRecord(c->ev_p2, fs));
       HFX_CUDA_TRY(cudaStreamWaitEvent(st, c->ev_p2, 0));
     }
-    if (!energy_only) {
+    for (int b = S.group_begin[q]; b < S.group_begin[q + 1] && !energy_only; ++b) {
       e0 = mark(st);
       const int nd = S.dense_begin[b + 1] - S.dense_begin[b];
       const int ng = S.generic_begin[b + 1] - S.generic_begin[b];
       if (nd > 0 && ct && S.b == 8 && dense_tma)  // [dense block pairs]
-        ct->y_acc_dense_tma(dim3(nzc, g.n1, nd), smem_dense_tma_ct(g.n1), st, tmW[b & 1], tmOrb, tmV,
+        ct->y_acc_dense_tma(dim3(nzc, g.n1, nd), smem_dense_tma_ct(g.n1), st, tmW[q & 1], tmOrb, tmV,
                             (const unsigned*)(couples + S.max_total_couples), n_orb,
                             S.d_dense_slots + S.dense_begin[b], S.d_slot_couple_base, S.d_slot_blocks, c0,
                             (const float2*)c->d_twct, vscale, c->d_err, (flags & HFX_TEST_STALL) ? 1 : 0);
@@ -1201,7 +1213,7 @@ static hfx_status run_passes(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
                                  gen_cap_max(c));
       if (ng > 0) close(kProfAccGeneric, e0, st);
     }
-    if (pipe) HFX_CUDA_TRY(cudaEventRecord(c->ev_p3[b & 1], st));
+    if (pipe) HFX_CUDA_TRY(cudaEventRecord(c->ev_p3[q & 1], st));
   }
   return HFX_OK;
 }
@@ -1684,7 +1696,7 @@ extern "C" hfx_status hfx_plan_stats(const hfx_ctx* c, int32_t n_orb, int64_t n_
   const bool eo = (flags & HFX_ENERGY_ONLY) != 0;
   long long launches = 0;
   if (n_pairs > 0) {
-    launches = 1 /* staging */ + (n_pairs > kPlaceHere) /* placement */ + 1 /* energy, widening */ + (long long)S.nbatches * 2;
+    launches = 1 /* staging */ + (n_pairs > kPlaceHere) /* placement */ + 1 /* energy, widening */ + (long long)S.ngroups * 2;
     if (!eo)
       for (int b = 0; b < S.nbatches; ++b)
         launches += (S.dense_begin[b + 1] > S.dense_begin[b]) + (S.generic_begin[b + 1] > S.generic_begin[b]) +
@@ -1802,6 +1814,7 @@ extern "C" hfx_status hfx_apply_noalloc(hfx_ctx* c, const void* orbitals, int32_
   // space left: the schedule is rebuilt with that transform budget when the default one does
   // not fit, and the call is refused only when a single block pair's transforms do not.
   Schedule S = make_host_schedule(c, n_orb);
+  build_groups(S, 0);  // the smallest transform buffer
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off += align256(std::max<size_t>(bytes, 16)); return o; };
   const size_t o_blocks = take(S.slot_blocks.size() * sizeof(int2));
@@ -1821,6 +1834,7 @@ extern "C" hfx_status hfx_apply_noalloc(hfx_ctx* c, const void* orbitals, int32_
     if (room >= (size_t)cap_max * couple_bytes + 256) {
       build_schedule(S, n_orb, c->bsize, room - 256, couple_bytes, dense_available(c), diag_available(c),
                      ragged_dense(c));
+      build_groups(S, 0);
       L = layout_of(c, S, n_orb, false);
     }
   }

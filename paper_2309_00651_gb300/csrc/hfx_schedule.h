@@ -27,6 +27,11 @@ struct Schedule {
   std::vector<int> dense_slots, generic_slots, diag_slots;  // concatenated over batches
   std::vector<int> dense_begin, generic_begin, diag_begin;  // [nbatches + 1] offsets into the lists
   bool ragged_rows = false;             // layout of ragged off-diagonal block pairs (build_schedule)
+  // consecutive batches whose forward and x passes run as one launch each (build_groups): group q is
+  // batches group_begin[q] .. group_begin[q + 1] - 1
+  std::vector<int> group_begin;
+  int ngroups = 0;
+  long long max_group_couples = 0;
   long long max_batch_couples = 0, max_total_couples = 0;
   // device copies
   int2* d_slot_blocks = nullptr;
@@ -130,6 +135,25 @@ static void build_schedule(Schedule& S, int n_orb, int b, size_t transform_budge
     S.generic_begin.push_back((int)S.generic_slots.size());
     S.diag_begin.push_back((int)S.diag_slots.size());
   }
+}
+
+// Groups of consecutive batches whose transforms together take at most `couples` (a batch that alone takes
+// more is a group): the forward and x passes run once a group, the accumulate passes batch by batch.
+static void build_groups(Schedule& S, long long couples) {
+  S.group_begin.assign(1, 0);
+  S.max_group_couples = 0;
+  long long in_group = 0;
+  for (int b = 0; b < S.nbatches; ++b) {
+    const long long n = S.slot_couple_base[S.batch_slot_begin[b + 1]] - S.slot_couple_base[S.batch_slot_begin[b]];
+    if (b > S.group_begin.back() && in_group + n > couples) {
+      S.group_begin.push_back(b);
+      in_group = 0;
+    }
+    in_group += n;
+    S.max_group_couples = std::max(S.max_group_couples, in_group);
+  }
+  S.group_begin.push_back(S.nbatches);
+  S.ngroups = (int)S.group_begin.size() - 1;
 }
 
 }  // namespace hfx
