@@ -27,21 +27,36 @@ namespace sinr {
 
 namespace {
 
-constexpr int kThreads = 256;
+// Threads per block: the FP64 pipe takes two operations a clock and SM, so a small system (1152 degrees of
+// freedom of 128 H2O) is spread over as many SMs as it has warps, and only a large one uses full blocks.
+// With 256 threads and the chain in local memory an update A of 1152 degrees of freedom (chain 4, three
+// factors) took 31 us, of 20000 31; now 15 and 23.  Large systems are bound by the FP64 pipe as before
+// (10^6: 697 us).
+constexpr int kSms = 152;
+constexpr int kMaxThreads = 256;
+int block_threads(long long n) {
+  const long long t = (n + kSms - 1) / kSms;
+  return (int)(t >= kMaxThreads ? kMaxThreads : (t + 31) / 32 * 32);
+}
 
 // per Suzuki-Yoshida factor k: c = Delta_k / (4 Q2) and hd = -Delta_k / 2
 struct SubSteps {
   double c[5], hd[5];
 };
 
-__global__ void __launch_bounds__(kThreads) k_update_n(SinrArgs a, long long n_dof, int n_res, int n_sy, SubSteps ss,
+// CL: the chain length at compile time (the chain then stays in registers and its exponentials overlap),
+// 0: read from the arguments
+template <int CL>
+__global__ void __launch_bounds__(kMaxThreads) k_update_n(SinrArgs a, long long n_dof, int n_res, int n_sy, SubSteps ss,
                                                        double sqrt_lam, double cq, const double* __restrict__ mass,
                                                        double* __restrict__ V, double* __restrict__ v1,
                                                        double* __restrict__ v2) {
-  const long long I = (long long)blockIdx.x * kThreads + threadIdx.x;
+  const long long I = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (I >= n_dof) return;
-  const int L = a.L;
-  double x1[kMaxChain], x2[kMaxChain];
+  const int L = CL ? CL : a.L;
+  constexpr int ML = CL ? CL : kMaxChain;
+  double x1[ML], x2[ML];
+#pragma unroll
   for (int j = 0; j < L; ++j) {
     x1[j] = v1[I * L + j];
     x2[j] = v2[I * L + j];
@@ -52,33 +67,36 @@ __global__ void __launch_bounds__(kThreads) k_update_n(SinrArgs a, long long n_d
     for (int k = 0; k < n_sy; ++k) {
       const double c = ss.c[k], hd = ss.hd[k];
       // e_j = exp(-v2_j Delta/2) serves both the rescaling of v1 and, squared, the denominator of H
-      double e[kMaxChain];
+      double e[ML];
       double den = M * vel * vel;
-      for (int j = 0; j < L; ++j) {
+    #pragma unroll
+  for (int j = 0; j < L; ++j) {
         x2[j] += c * fma(a.Q1 * x1[j], x1[j], -a.kT);
         e[j] = exp(hd * x2[j]);
         den += cq * (x1[j] * x1[j]) * (e[j] * e[j]);
       }
       const double H = sqrt_lam * rsqrt(den);
       vel *= H;
-      for (int j = 0; j < L; ++j) {
+    #pragma unroll
+  for (int j = 0; j < L; ++j) {
         x1[j] *= H * e[j];
         x2[j] += c * fma(a.Q1 * x1[j], x1[j], -a.kT);
       }
     }
   }
   V[I] = vel;
+#pragma unroll
   for (int j = 0; j < L; ++j) {
     v1[I * L + j] = x1[j];
     v2[I * L + j] = x2[j];
   }
 }
 
-__global__ void __launch_bounds__(kThreads) k_update_v(SinrArgs a, long long n_dof, double dt, double inv_lam,
+__global__ void __launch_bounds__(kMaxThreads) k_update_v(SinrArgs a, long long n_dof, double dt, double inv_lam,
                                                        const double* __restrict__ mass, const double* __restrict__ force,
                                                        const double* __restrict__ force_extra, double* __restrict__ V,
                                                        double* __restrict__ v1) {
-  const long long I = (long long)blockIdx.x * kThreads + threadIdx.x;
+  const long long I = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (I >= n_dof) return;
   const int L = a.L;
   const double M = mass[I], inv_m = 1.0 / M;
@@ -105,18 +123,18 @@ __global__ void __launch_bounds__(kThreads) k_update_v(SinrArgs a, long long n_d
   for (int j = 0; j < L; ++j) v1[I * L + j] *= inv;
 }
 
-__global__ void __launch_bounds__(kThreads) k_update_x(SinrArgs a, long long n_dof, double dt, double decay,
+__global__ void __launch_bounds__(kMaxThreads) k_update_x(SinrArgs a, long long n_dof, double dt, double decay,
                                                        double noise, const double* __restrict__ V,
                                                        double* __restrict__ X, double* __restrict__ v2,
                                                        const double* __restrict__ R) {
-  const long long I = (long long)blockIdx.x * kThreads + threadIdx.x;
+  const long long I = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (I >= n_dof) return;
   X[I] += V[I] * dt;
   const int L = a.L;
   for (int j = 0; j < L; ++j) v2[I * L + j] = v2[I * L + j] * decay + noise * R[I * L + j];
 }
 
-int blocks(long long n) { return (int)((n + kThreads - 1) / kThreads); }
+int blocks(long long n, int threads) { return (int)((n + threads - 1) / threads); }
 
 }  // namespace
 
@@ -130,14 +148,26 @@ cudaError_t update_n(const SinrArgs& a, long long n_dof, double dt, int n_res, c
     ss.hd[k] = -0.5 * delta;
   }
   const double sqrt_lam = sqrt(a.L * a.kT), cq = (double)a.L / (a.L + 1.0) * a.Q1;
-  k_update_n<<<blocks(n_dof), kThreads, 0, st>>>(a, n_dof, n_res, n_sy, ss, sqrt_lam, cq, mass, V, v1, v2);
+  const int t = block_threads(n_dof), b = blocks(n_dof, t);
+#define HFX_SINR_N(CL) k_update_n<CL><<<b, t, 0, st>>>(a, n_dof, n_res, n_sy, ss, sqrt_lam, cq, mass, V, v1, v2)
+  switch (a.L) {
+    case 1: HFX_SINR_N(1); break;
+    case 2: HFX_SINR_N(2); break;
+    case 3: HFX_SINR_N(3); break;
+    case 4: HFX_SINR_N(4); break;
+    case 5: HFX_SINR_N(5); break;
+    case 6: HFX_SINR_N(6); break;
+    default: HFX_SINR_N(0); break;
+  }
+#undef HFX_SINR_N
   return cudaGetLastError();
 }
 
 cudaError_t update_v(const SinrArgs& a, long long n_dof, double dt, const double* mass, const double* force,
                      const double* force_extra, double* V, double* v1, cudaStream_t st) {
   if (n_dof == 0) return cudaSuccess;
-  k_update_v<<<blocks(n_dof), kThreads, 0, st>>>(a, n_dof, dt, 1.0 / (a.L * a.kT), mass, force, force_extra, V, v1);
+  const int t = block_threads(n_dof);
+  k_update_v<<<blocks(n_dof, t), t, 0, st>>>(a, n_dof, dt, 1.0 / (a.L * a.kT), mass, force, force_extra, V, v1);
   return cudaGetLastError();
 }
 
@@ -148,7 +178,8 @@ cudaError_t update_x(const SinrArgs& a, long long n_dof, double dt, const double
   const double decay = exp(-a.gamma * dt);
   const double sigma = sqrt(2.0 * a.kT * a.gamma / a.Q2);
   const double noise = sigma * sqrt((1.0 - exp(-2.0 * a.gamma * dt)) / (2.0 * a.gamma));
-  k_update_x<<<blocks(n_dof), kThreads, 0, st>>>(a, n_dof, dt, decay, noise, V, X, v2, R);
+  const int t = block_threads(n_dof);
+  k_update_x<<<blocks(n_dof, t), t, 0, st>>>(a, n_dof, dt, decay, noise, V, X, v2, R);
   return cudaGetLastError();
 }
 
