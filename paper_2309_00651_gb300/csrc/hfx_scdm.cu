@@ -26,9 +26,33 @@ namespace ace {
 
 namespace {
 
-constexpr int kUpdThreads = 256;
-constexpr int kUpdPoints = 4;  // grid points per thread per sweep (independent dot products)
-constexpr int kUpdBlocksPerSm = 3;  // resident update blocks per SM at its launch bounds
+constexpr int kUpdThreads = 128;
+constexpr int kUpdBlocksPerSm = 5;  // resident update blocks per SM at its launch bounds
+// grid points and orbital rows a thread of the update has in flight: FP32 waits for memory and keeps one
+// point's rows in flight; FP64 also for its pipe, whose latency four independent points hide
+template <typename T> struct UpdShape {
+  static constexpr int points = sizeof(T) == 4 ? 1 : 4, rows = sizeof(T) == 4 ? 64 : 8;
+};
+constexpr int kInitThreads = 256;
+constexpr int kUpdRounds = 4;
+constexpr size_t kL2Keep = size_t(64) << 20;
+
+// launch whose start may overlap the kernel before it on the stream: the kernel itself waits
+// (cudaGridDependencySynchronize) before it touches what that kernel writes
+template <typename... P, typename... A>
+cudaError_t launch_overlapped(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 
 template <typename T>
 __device__ __forceinline__ T round_to(double v);
@@ -97,14 +121,14 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // residual norms nu_p = |Psi^T[:, p]|^2 (in the compute type, widened), the FP32 copy of the
 // orbitals when T = float, and the per-block maxima
 template <typename T>
-__global__ void __launch_bounds__(kUpdThreads) k_scdm_init(const double* __restrict__ psi, long long N, int n,
+__global__ void __launch_bounds__(kInitThreads) k_scdm_init(const double* __restrict__ psi, long long N, int n,
                                                            T* __restrict__ a32, double* __restrict__ nu,
                                                            double* __restrict__ bmax, long long* __restrict__ bidx) {
   __shared__ double sv[32];
   __shared__ long long si[32];
   double best = -2.0;
   long long bi = (long long)1 << 62;
-  for (long long p = (long long)blockIdx.x * kUpdThreads + threadIdx.x; p < N; p += (long long)gridDim.x * kUpdThreads) {
+  for (long long p = (long long)blockIdx.x * kInitThreads + threadIdx.x; p < N; p += (long long)gridDim.x * kInitThreads) {
     T acc = T(0);
     for (int i = 0; i < n; ++i) {
       const T v = round_to<T>(psi[(long long)i * N + p]);
@@ -153,6 +177,9 @@ __global__ void __launch_bounds__(kPickThreads, 1) k_scdm_pick(const double* __r
   // whole 16-byte pieces, which stay inside the row
   T* qs = reinterpret_cast<T*>((reinterpret_cast<uintptr_t>(hp + 32 * n) + 15) & ~uintptr_t(15));
   const T* Q = QS ? qs : qt;
+  // q_0 .. q_{j-1} are there (the update before this kernel let it start after its own wait for them); the
+  // maxima and the residual norms are not
+  cudaTriggerProgrammaticLaunchCompletion();
   if (QS && j > 0) {
     constexpr int EPC = 16 / (int)sizeof(T);
     const int cpr = (j + EPC - 1) / EPC;
@@ -161,6 +188,7 @@ __global__ void __launch_bounds__(kPickThreads, 1) k_scdm_pick(const double* __r
       cp_async16(qs + (long long)i * ldt + kc * EPC, qt + (long long)i * ldt + kc * EPC);
     }
   }
+  cudaGridDependencySynchronize();
   {  // argmax over the per-block maxima (lowest index on a tie), the whole block
     double best = -2.0;
     long long bi = (long long)1 << 62;
@@ -267,51 +295,73 @@ __global__ void __launch_bounds__(kPickThreads, 1) k_scdm_pick(const double* __r
   }
 }
 
-// step j: c_p = q_j . Psi^T[:, p], nu_p -= c_p^2 (picked points stay at -1), per-block maxima;
-// each thread takes kUpdPoints grid points, rows unrolled for loads in flight
+// step j: c_p = q_j . Psi^T[:, p], nu_p -= c_p^2 (picked points stay at -1), per-block maxima; UpdShape
+// points per thread and rows in flight.
+//
+// A step streams all of Psi (191 MB for 128 FP32 orbitals on 72^3) and does next to no arithmetic, so
+// bandwidth bounds it.  Psi exceeds L2 but not by much, and an even step takes its runs of grid points
+// (`run` of them per block and round) from first to last, an odd one from last to first: each step begins
+// with what the one before left in L2; the dot products and the picks do not depend on the order of the
+// points.  A round is a chain of n / rows load latencies, so few rounds and many rows in flight win:
+// 128 orbitals on 72^3, whole localisation, 4 points a thread and no order 7.79 ms; 4 rounds with 16, 32,
+// 64 rows 7.25, 6.72, 5.93; 6 and 8 rounds lose.  The launches overlap (see launch_overlapped): 48 orbitals
+// on 48^3, which fits L2, 1.25 -> 1.04 ms, 20 on 32^3 0.40 -> 0.33.
 template <typename T>
 __global__ void __launch_bounds__(kUpdThreads, kUpdBlocksPerSm) k_scdm_update(const T* __restrict__ A, long long N, int n,
-                                                             const T* __restrict__ qt, long long ldt, int j,
-                                                             const long long* __restrict__ piv,
+                                                             const T* __restrict__ qt, long long ldt, int j, int run,
+                                                             int rounds, const long long* __restrict__ piv,
                                                              double* __restrict__ nu, double* __restrict__ bmax,
                                                              long long* __restrict__ bidx) {
   extern __shared__ __align__(16) unsigned char smem[];
   T* q = reinterpret_cast<T*>(smem);  // [n]
   __shared__ double sv[32];
   __shared__ long long si[32];
+  cudaGridDependencySynchronize();  // the pick of this step
+  // only now: the next pick, which this lets start, reads q_0 .. q_j before it waits for this kernel
+  cudaTriggerProgrammaticLaunchCompletion();
   for (int i = threadIdx.x; i < n; i += blockDim.x) q[i] = qt[(long long)i * ldt + j];
   __syncthreads();
   const long long picked = piv[j];
   double best = -2.0;
   long long bi = (long long)1 << 62;
-  // block b takes the contiguous run [b chunk, (b+1) chunk) of grid points (chunk a multiple of
-  // 32), in sweeps of kUpdThreads x kUpdPoints points: every block gets the same share
-  const long long chunk = ((N + gridDim.x - 1) / gridDim.x + 31) / 32 * 32;
-  const long long b0 = (long long)blockIdx.x * chunk;
-  const long long b1 = min(N, b0 + chunk);
-  for (long long p0 = b0 + threadIdx.x; p0 < b1; p0 += (long long)kUpdThreads * kUpdPoints) {
-    T c[kUpdPoints];
-    bool in[kUpdPoints];
+  for (int r = 0; r < rounds; ++r) {
+    const int rr = (j & 1) ? rounds - 1 - r : r;
+    const long long p0 = ((long long)rr * gridDim.x + blockIdx.x) * run + threadIdx.x;
+    constexpr int kPts = UpdShape<T>::points, kRows = UpdShape<T>::rows;
+    bool in[kPts];
+    double old[kPts];
+    T c[kPts];
 #pragma unroll
-    for (int u = 0; u < kUpdPoints; ++u) {
-      c[u] = T(0);
-      in[u] = p0 + u * kUpdThreads < b1;
+    for (int k = 0; k < kPts; ++k) {
+      in[k] = (int)threadIdx.x + k * kUpdThreads < run && p0 + k * kUpdThreads < N;
+      old[k] = in[k] ? nu[p0 + k * kUpdThreads] : -1.0;
+      c[k] = T(0);
+    }
+    if (!in[0]) continue;
+    const T* row = A + p0;
+    int i = 0;
+    for (; i + kRows <= n; i += kRows) {
+      T v[kRows][kPts];
+#pragma unroll
+      for (int u = 0; u < kRows; ++u)
+#pragma unroll
+        for (int k = 0; k < kPts; ++k) v[u][k] = in[k] ? row[(long long)(i + u) * N + k * kUpdThreads] : T(0);
+#pragma unroll
+      for (int u = 0; u < kRows; ++u)
+#pragma unroll
+        for (int k = 0; k < kPts; ++k) c[k] = fma(q[i + u], v[u][k], c[k]);
     }
 #pragma unroll 8
-    for (int i = 0; i < n; ++i) {
-      const T qi = q[i];
-      const T* row = A + (long long)i * N + p0;
+    for (; i < n; ++i)
 #pragma unroll
-      for (int u = 0; u < kUpdPoints; ++u)
-        if (in[u]) c[u] = fma(qi, row[u * kUpdThreads], c[u]);
-    }
+      for (int k = 0; k < kPts; ++k)
+        if (in[k]) c[k] = fma(q[i], row[(long long)i * N + k * kUpdThreads], c[k]);
 #pragma unroll
-    for (int u = 0; u < kUpdPoints; ++u) {
-      const long long p = p0 + u * kUpdThreads;
-      if (!in[u]) continue;
-      const double old = nu[p];
-      const double cc = (double)c[u];
-      const double v = (old < 0.0 || p == picked) ? -1.0 : old - cc * cc;
+    for (int k = 0; k < kPts; ++k) {
+      if (!in[k]) continue;
+      const long long p = p0 + k * kUpdThreads;
+      const double cc = (double)c[k];
+      const double v = (old[k] < 0.0 || p == picked) ? -1.0 : old[k] - cc * cc;
       nu[p] = v;
       take_max(best, bi, v, p);
     }
@@ -320,9 +370,8 @@ __global__ void __launch_bounds__(kUpdThreads, kUpdBlocksPerSm) k_scdm_update(co
   if (threadIdx.x == 0) { bmax[blockIdx.x] = best; bidx[blockIdx.x] = bi; }
 }
 
-// blocks of the init / update launches: one wave of kUpdBlocksPerSm blocks on every SM (equal
-// shares of the grid, so no SM runs a block more than the others), fewer for small grids (at
-// least kUpdThreads points per block)
+// blocks of the init / update launches: one wave of kUpdBlocksPerSm blocks on every SM, fewer for small
+// grids (at least kUpdThreads points per block)
 static int scdm_blocks(long long N, int sm_count) {
   const long long cover = (N + kUpdThreads - 1) / kUpdThreads;
   return (int)std::max(1LL, std::min<long long>(cover, (long long)sm_count * kUpdBlocksPerSm));
@@ -334,7 +383,7 @@ static cudaError_t scdm_run(const double* psi, long long N, int n, T* a32, doubl
                             cudaStream_t st) {
   const int nb = scdm_blocks(N, sm_count);
   const T* A = a32 ? a32 : reinterpret_cast<const T*>(psi);
-  k_scdm_init<T><<<nb, kUpdThreads, 0, st>>>(psi, N, n, a32, nu, bmax, bidx);
+  k_scdm_init<T><<<nb, kInitThreads, 0, st>>>(psi, N, n, a32, nu, bmax, bidx);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const size_t base_smem = 34 * (size_t)n * sizeof(T);
@@ -347,13 +396,20 @@ static cudaError_t scdm_run(const double* psi, long long N, int n, T* a32, doubl
     if (e != cudaSuccess) return e;
   }
   const size_t upd_smem = (size_t)n * sizeof(T);
+  // runs of a multiple of 8 points (whole 32-byte sectors), as few rounds as kUpdThreads allows, but several
+  // where Psi exceeds L2 and the last rounds of a step are what the next one finds there
+  const long long per_block = (N + nb - 1) / nb, most = (long long)kUpdThreads * UpdShape<T>::points;
+  int rounds = (int)std::max<long long>(1, (per_block + most - 1) / most);
+  if (UpdShape<T>::points == 1 && (size_t)n * N * sizeof(T) > kL2Keep)
+    rounds = (int)std::max<long long>(rounds, std::min<long long>(kUpdRounds, per_block / 32));
+  const int run = (int)std::min<long long>(most, ((per_block + rounds - 1) / rounds + 7) / 8 * 8);
+  rounds = (int)((N + (long long)nb * run - 1) / ((long long)nb * run));
   for (int j = 0; j < n; ++j) {
-    if (qs)
-      k_scdm_pick<T, true><<<1, kPickThreads, pick_smem, st>>>(psi, N, n, j, bmax, bidx, nb, piv, qt, q64, ldt, rdiag, err);
-    else
-      k_scdm_pick<T, false><<<1, kPickThreads, pick_smem, st>>>(psi, N, n, j, bmax, bidx, nb, piv, qt, q64, ldt, rdiag, err);
-    if (j + 1 < n) k_scdm_update<T><<<nb, kUpdThreads, upd_smem, st>>>(A, N, n, qt, ldt, j, piv, nu, bmax, bidx);
-    e = cudaGetLastError();
+    e = launch_overlapped(qs ? k_scdm_pick<T, true> : k_scdm_pick<T, false>, 1, kPickThreads, pick_smem, st, psi, N, n, j,
+                          bmax, bidx, nb, piv, qt, q64, ldt, rdiag, err);
+    if (e == cudaSuccess && j + 1 < n)
+      e = launch_overlapped(k_scdm_update<T>, nb, kUpdThreads, upd_smem, st, A, N, n, qt, ldt, j, run, rounds, piv, nu,
+                            bmax, bidx);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
