@@ -911,13 +911,22 @@ __global__ void __launch_bounds__(256) k_stage(uint4* __restrict__ zero, long lo
   } else {
     for (long long i = first; i < table_words; i += step) table[i] = -1;
   }
-  for (long long i = first; i < nzero; i += step) zero[i] = make_uint4(0u, 0u, 0u, 0u);
+  constexpr int U = 4;  // pieces a thread has in flight
   if (src)
-    for (long long i = first; i < n / 4; i += step) {  // (three even edges: n is a multiple of 8)
-      const double2 u = __ldcs(reinterpret_cast<const double2*>(src) + 2 * i);
-      const double2 v = __ldcs(reinterpret_cast<const double2*>(src) + 2 * i + 1);
-      reinterpret_cast<float4*>(dst)[i] = make_float4((float)u.x, (float)u.y, (float)v.x, (float)v.y);
+    for (long long i = first; i < n / 4; i += U * step) {  // (three even edges: n is a multiple of 8)
+      double2 a[U], b[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (i + u * step < n / 4) {
+          a[u] = __ldcs(reinterpret_cast<const double2*>(src) + 2 * (i + u * step));
+          b[u] = __ldcs(reinterpret_cast<const double2*>(src) + 2 * (i + u * step) + 1);
+        }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (i + u * step < n / 4)
+          reinterpret_cast<float4*>(dst)[i + u * step] = make_float4((float)a[u].x, (float)a[u].y, (float)b[u].x, (float)b[u].y);
     }
+  for (long long i = first; i < nzero; i += step) zero[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // E_x = scale * sum_g w_g sum_y epart[g][y] by the first `ne` blocks of the call's last launch: block b
@@ -927,9 +936,7 @@ __global__ void __launch_bounds__(256) k_stage(uint4* __restrict__ zero, long lo
 // accumulator, exactly and with integer operations (FP32 subnormals flush to zero); n is a multiple of 4
 constexpr int kEnergyBlocks = 63;
 
-__device__ __forceinline__ void widen_v4(const float* __restrict__ v32, double* __restrict__ v, long long i4,
-                                         int accumulate) {
-  const float4 a = __ldcs(reinterpret_cast<const float4*>(v32) + i4);
+__device__ __forceinline__ void widen_v4(const float4 a, double* __restrict__ v, long long i4, int accumulate) {
   double2 lo = make_double2(ct::widen_exact(a.x), ct::widen_exact(a.y));
   double2 hi = make_double2(ct::widen_exact(a.z), ct::widen_exact(a.w));
   double2* d = reinterpret_cast<double2*>(v) + 2 * i4;
@@ -947,9 +954,17 @@ __global__ void __launch_bounds__(256) k_finish(const double* __restrict__ epart
                                                 double* __restrict__ ex, const float* __restrict__ v32,
                                                 double* __restrict__ v, long long n) {
   if ((int)blockIdx.x >= ne) {
-    for (long long i = (blockIdx.x - ne) * (long long)blockDim.x + threadIdx.x; i < n / 4;
-         i += (long long)(gridDim.x - ne) * blockDim.x)
-      widen_v4(v32, v, i, accumulate);
+    const long long step = (long long)(gridDim.x - ne) * blockDim.x;
+    constexpr int U = 4;  // pieces a thread has in flight
+    for (long long i = (blockIdx.x - ne) * (long long)blockDim.x + threadIdx.x; i < n / 4; i += U * step) {
+      float4 a[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (i + u * step < n / 4) a[u] = __ldcs(reinterpret_cast<const float4*>(v32) + i + u * step);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (i + u * step < n / 4) widen_v4(a[u], v, i + u * step, accumulate);
+    }
     return;
   }
   __shared__ double red[32];

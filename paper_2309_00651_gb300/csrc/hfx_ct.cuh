@@ -187,6 +187,41 @@ __device__ __forceinline__ double widen_exact(float v) {
   return __hiloint2double((int)hi, (int)lo);
 }
 
+// (s, e) += (a, ea): the rounding error of s + a goes to e (Knuth's two-sum)
+__device__ __forceinline__ void two_sum(float& s, float& e, float a, float ea) {
+  const float t = __fadd_rn(s, a), b = __fsub_rn(t, s);
+  e += __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(a, b)) + ea;
+  s = t;
+}
+
+// Sum of one value per thread over a block for the plane energies: a tree per warp into red, then one over
+// the warps.  FP32 trees for the edges where that was measured to be enough (E within 2e-7); the others,
+// whose planes the runtime-geometry pass sums in FP64, carry the rounding errors along (about 48 bits),
+// which costs the x pass 1 to 3%.
+template <int N> struct PlaneSum {
+  static constexpr bool compensated = !(N == 32 || N == 48 || N == 64 || N == 72 || N == 80 || N == 90 || N == 96 || N == 128);
+  static __device__ __forceinline__ void warp(float s, float2* red) {
+    float e = 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      if constexpr (compensated) two_sum(s, e, __shfl_down_sync(0xffffffffu, s, o), __shfl_down_sync(0xffffffffu, e, o));
+      else s += __shfl_down_sync(0xffffffffu, s, o);
+    }
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_float2(s, e);
+  }
+  // by the threads of warp 0
+  template <int NW> static __device__ __forceinline__ void block(const float2* red, double* out) {
+    float2 r = threadIdx.x < NW ? red[threadIdx.x] : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int o = NW > 16 ? 16 : NW > 8 ? 8 : NW > 4 ? 4 : NW > 2 ? 2 : 1; o > 0; o >>= 1) {
+      if constexpr (compensated)
+        two_sum(r.x, r.y, __shfl_down_sync(0xffffffffu, r.x, o), __shfl_down_sync(0xffffffffu, r.y, o));
+      else r.x += __shfl_down_sync(0xffffffffu, r.x, o);
+    }
+    if (threadIdx.x == 0) *out = compensated ? widen_exact(r.x) + widen_exact(r.y) : widen_exact(r.x);
+  }
+};
+
 constexpr int kUnroll = 4;
 
 // threads per block of the compile-time plane kernels: 256, but 512 where the padded plane is so
@@ -302,12 +337,12 @@ k_fwd_yz_ct(const T* __restrict__ orb, long long Ntot, const int4* __restrict__ 
 // ----------------------------------------------------------------------------------
 // pass 2: forward FFT along x, Coulomb multiply + energy, inverse along x and z
 // ----------------------------------------------------------------------------------
-// one item (couple cl = it / N, y-plane y = it mod N); red: [2][32] floats of shared memory used
+// one item (couple cl = it / N, y-plane y = it mod N); red: [2][32] pairs of floats in shared memory used
 // alternately (par) by consecutive items of a block
 template <typename T, int N>
 __device__ __forceinline__ void x_coulomb_ct_item(const int4* __restrict__ couples, int c0, cx<T>* __restrict__ W,
                                                   const T* __restrict__ vtab, double* __restrict__ epart,
-                                                  int energy_only, cx<T>* buf, const cx<T>* tw, float (*red)[32],
+                                                  int energy_only, cx<T>* buf, const cx<T>* tw, float2 (*red)[32],
                                                   int par, int it) {
   using C = cx<T>;
   constexpr int S = N + 1, PLANE = N * N, NT = PlaneThreads<N>::value;
@@ -356,23 +391,11 @@ __device__ __forceinline__ void x_coulomb_ct_item(const int4* __restrict__ coupl
     }
   }
   static_assert(sizeof(T) == 4, "compile-time passes are FP32");
-  // block sum without barriers of its own: a shuffle tree per warp, the warp partials to
-  // red[par] now, and warp 0 adds them (a second tree) after the barrier that the inverse
-  // stages need anyway
-  {
-    float v = e_acc;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) red[par][threadIdx.x >> 5] = v;
-  }
+  // block sum without barriers of its own: the warps' sums to red[par] now, and warp 0 adds them after the
+  // barrier that the inverse stages need anyway
+  PlaneSum<N>::warp(e_acc, red[par]);
   __syncthreads();
-  if (threadIdx.x < 32) {
-    constexpr int NW = (NT + 31) / 32;
-    float r = threadIdx.x < NW ? red[par][threadIdx.x] : 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
-    if (threadIdx.x == 0) epart[(long long)(c0 + cl) * N + y] = widen_exact(r);
-  }
+  if (threadIdx.x < 32) PlaneSum<N>::template block<(NT + 31) / 32>(red[par], epart + (long long)(c0 + cl) * N + y);
   if (energy_only) return;
   // inverse transforms along different axes commute: z first (rows), then the remaining x
   // stages, the last of which writes W directly
@@ -391,7 +414,7 @@ k_x_coulomb_ct(const int4* __restrict__ couples, int c0, int c1, cx<T>* __restri
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
   C* tw = buf + N * S;
-  __shared__ float red[2][32];  // warp partials of the plane energy, double-buffered by item parity
+  __shared__ float2 red[2][32];  // warp partials of the plane energy, double-buffered by item parity
   for (int i = threadIdx.x; i < P.twtotal; i += PlaneThreads<N>::value) tw[i] = twg[i];
   int par = 0;
   const int items = (c1 - c0) * N;

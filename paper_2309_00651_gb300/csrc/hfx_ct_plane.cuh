@@ -257,11 +257,11 @@ k_fwd_plane(const float* __restrict__ orb, long long Ntot, const int4* __restric
 // ----------------------------------------------------------------------------------
 // x pass: forward x, Coulomb multiply and energy, inverse x and z of y-plane y of couple cl
 // ----------------------------------------------------------------------------------
-// red: [2][32] floats of shared memory used alternately (par) by consecutive items of a block
+// red: [2][32] pairs of floats in shared memory used alternately (par) by consecutive items of a block
 template <int N, int NT>
 __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, const float* __restrict__ vtab,
                                              double* __restrict__ epart, int energy_only, cpair* buf,
-                                             const cpair* tw, float (*red)[32], int par, int cl, int y) {
+                                             const cpair* tw, float2 (*red)[32], int par, int cl, int y) {
   using G = PlaneGeo<N>;
   constexpr int R = G::R, S = G::SX, PLANE = N * N;
   float2* wc = W + ((long long)cl * N + y) * PLANE;
@@ -284,8 +284,8 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
     for (int k = 0; k < R; ++k) p[G::place(k) * (4 * S) + 2 * ((G::place(k) >> 1) & 1)] = v[k];
   }
   // the tile x = 4 X .. 4 X + 3, z = 4 Z .. 4 Z + 3: last forward x stage, v(G) and the energy, first
-  // inverse x stage, first inverse z stage.  The plane's energy in FP32 (a few terms per thread, a tree
-  // per warp, then over the block), widened once; planes and couples are summed in FP64
+  // inverse x stage, first inverse z stage.  The plane's energy: a few tiles' terms per thread in FP32,
+  // then PlaneSum over the block; planes and couples are summed in FP64
   float e_acc = 0.f;
   const float* vy = vtab + (long long)y * N;
   __syncthreads();
@@ -335,22 +335,14 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
       }
     }
   }
-  // block sum without barriers of its own: a shuffle tree per warp, the warp partials to red[par] now,
-  // and warp 0 adds them (a second tree) after the barrier that the inverse stages need anyway
-  {
-    float v = e_acc;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) red[par][threadIdx.x >> 5] = v;
-  }
+  // block sum without barriers of its own: the warps' sums to red[par] now, and warp 0 adds them after the
+  // barrier that the inverse stages need anyway -- at the end of the item, when no other warp waits for it,
+  // unless the block has its SM to itself (128^3: 9.63 against 9.82 ms at the end)
+  constexpr bool kLate = NT < 480;
+  PlaneSum<N>::warp(e_acc, red[par]);
   __syncthreads();
-  if (threadIdx.x < 32) {
-    constexpr int NW = NT / 32;
-    float r = threadIdx.x < NW ? red[par][threadIdx.x] : 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
-    if (threadIdx.x == 0) epart[(long long)(c0 + cl) * N + y] = widen_exact(r);
-  }
+  double* ep = epart + (long long)(c0 + cl) * N + y;
+  if (threadIdx.x < 32 && (!kLate || energy_only)) PlaneSum<N>::template block<NT / 32>(red[par], ep);
   if (energy_only) return;
   // inverse z: elements e + 4 k of row x
 #pragma unroll 1
@@ -381,6 +373,7 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
 #pragma unroll
     for (int k = 0; k < R; ++k) dst[k * (4 * N)] = v[k];
   }
+  if (kLate && threadIdx.x < 32) PlaneSum<N>::template block<NT / 32>(red[par], ep);
 }
 
 template <int N, int NT, int MINB>
@@ -392,7 +385,7 @@ k_x_plane(const int4* __restrict__ couples, int c0, int c1, float2* __restrict__
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpair* tw = reinterpret_cast<cpair*>(smem_raw);
   cpair* buf = tw + G::TW;
-  __shared__ float red[2][32];  // warp partials of the plane energy, double-buffered by item parity
+  __shared__ float2 red[2][32];  // warp partials of the plane energy, double-buffered by item parity
   for (int i = threadIdx.x; i < G::TW; i += NT) tw[i] = cpair{twg[i].x, twg[i].y};
   int par = 0;
   const int items = (c1 - c0) * N;
