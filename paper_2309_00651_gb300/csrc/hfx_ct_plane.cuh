@@ -12,13 +12,16 @@
 // stage at a time takes four.  y keeps the split of stage_plan(N), which the accumulate passes invert.
 // Measured against the one-stage-at-a-time form, us per launch of 256 couples: forward / x pass 45 / 45
 // -> 28 / 27 (32^3), 108 / 127 -> 90 / 96 (48^3), 231 / 239 -> 194 / 221 (64^3), 338 / 409 -> 292 / 346
-// (72^3), 436 / 531 -> 415 / 472 (80^3), 778 / 1012 -> 726 / 892 (96^3), 2262 / 2872 -> 2075 / 2368
+// (72^3), 436 / 531 -> 415 / 472 (80^3), 778 / 1012 -> 676 / 892 (96^3), 2262 / 2872 -> 2075 / 2368
 // (128^3).  At 72^3 the x pass moves 4.4 TB/s of DRAM; with its loads and stores taken out it runs in
 // 252 us, with its shared-memory stages taken out in 254, so what is left is how far the two overlap.
 //
 // Layouts, chosen so that the half-warps of every stage touch 16 different 8-byte banks:
 //   forward: z = 4 D + e of row y sits at y S + e E + D (E = 4 or 12 mod 16, S = 3 mod 16): four rows x
-//            four e of the z stage, runs of D in the last stage, and runs of (D, e) in the y stage;
+//            four e of the z stage, runs of D in the last stage, and runs of (D, e) in the y stage.
+//            At 96^3 rows go without gaps (E = 24 = 8, S = 97 = 1 mod 16, eight rows x two e in the z stage,
+//            runs of places in the y stage), so that three planes fit an SM instead of two: 721 -> 676 us (at
+//            72^3 a fifth plane by rows without gaps lost, 288 -> 302 us);
 //   x pass:  (x, z) sits at x S + z + 2 ((x / 8) mod 2), S = N + 2 (2 or 10 mod 16): eight rows x two z
 //            in the z stage, runs of z in the x stages, and in the tile stage 16-byte accesses of which
 //            eight consecutive lanes (two x, four z tiles) cover all banks.
@@ -34,15 +37,27 @@ namespace ct {
 template <int N> struct PlaneGeo {
   static_assert(N % 4 == 0, "plane passes need an edge that is a multiple of 4");
   static constexpr int R = N / 4;                                   // large radix of z and x
-  static constexpr int E = (R + 3) / 8 * 8 + 4;                     // >= R, 4 mod 8
-  static constexpr int SF = 4 * E + 3;                              // forward row stride
+  // forward rows without gaps, where that lets another plane fit an SM
+  static constexpr bool kDense = R == 24;
+  static constexpr int E = kDense ? R : (R + 3) / 8 * 8 + 4;        // >= R, 4 mod 8
+  static constexpr int SF = 4 * E + (kDense ? 1 : 3);               // forward row stride
+  // row and z digit of task `id` of the z stage
+  static __device__ __forceinline__ void z_task(int id, int& y, int& e) {
+    if constexpr (kDense) {
+      e = (id >> 3) & 3;
+      y = (id >> 5) * 8 + (id & 7);
+    } else {
+      e = (id >> 2) & 3;
+      y = (id >> 4) * 4 + (id & 3);
+    }
+  }
   static constexpr int SX = N + 2;                                  // x-pass row stride
   static constexpr StagePlan Y = stage_plan(N);
   static_assert(Y.ns == 2, "two y stages");
   static constexpr int RY0 = Y.r[0], RY1 = Y.r[1];
   static constexpr int TW = 4 * (R + R % 2);                        // z and x twiddles, then y's
   static constexpr int TWY = RY1 * RY0;
-  static_assert(E >= R && E % 8 == 4, "bank-spreading stride of the z digits");
+  static_assert(E >= R && (kDense || E % 8 == 4), "bank-spreading stride of the z digits");
   // place of output k of the large radix among its R: as two radices the runtime-geometry kernels know
   // (plane_radices) would leave it, so that the tables and the pencil and batch kernels share the order
   static constexpr PlaneRadices P = plane_radices(R);
@@ -66,7 +81,7 @@ template <> struct PlaneCfg<60>  { static constexpr int fnt = 128, fmb = 5,  un 
 template <> struct PlaneCfg<64>  { static constexpr int fnt = 128, fmb = 5,  un = 4, xnt = 128, xmb = 6; };
 template <> struct PlaneCfg<72>  { static constexpr int fnt = 160, fmb = 4,  un = 3, xnt = 128, xmb = 5; };
 template <> struct PlaneCfg<80>  { static constexpr int fnt = 160, fmb = 4,  un = 4, xnt = 160, xmb = 4; };
-template <> struct PlaneCfg<96>  { static constexpr int fnt = 192, fmb = 2,  un = 6, xnt = 384, xmb = 2; };
+template <> struct PlaneCfg<96>  { static constexpr int fnt = 128, fmb = 3,  un = 6, xnt = 384, xmb = 2; };
 template <> struct PlaneCfg<100> { static constexpr int fnt = 224, fmb = 2,  un = 4, xnt = 256, xmb = 2; };
 template <> struct PlaneCfg<108> { static constexpr int fnt = 224, fmb = 2,  un = 4, xnt = 256, xmb = 2; };
 template <> struct PlaneCfg<120> { static constexpr int fnt = 480, fmb = 1,  un = 4, xnt = 480, xmb = 1; };
@@ -166,7 +181,8 @@ __device__ __forceinline__ void fwd_plane_item(const float* __restrict__ orb, lo
   // z: elements e + 4 k of row y
 #pragma unroll 1
   for (int id = threadIdx.x; id < 4 * N; id += NT) {
-    const int e = (id >> 2) & 3, y = (id >> 4) * 4 + (id & 3);
+    int y, e;
+    G::z_task(id, y, e);
     cpair* p = buf + y * S + e * E;
     cpair v[R];
 #pragma unroll
@@ -181,7 +197,7 @@ __device__ __forceinline__ void fwd_plane_item(const float* __restrict__ orb, lo
 #pragma unroll 1
   for (int id = threadIdx.x; id < RY1 * N; id += NT) {
     const int j = id / N, c = id - j * N;
-    cpair* p = buf + j * S + (c & 3) * E + (c >> 2);
+    cpair* p = buf + j * S + (G::kDense ? c : (c & 3) * E + (c >> 2));
     cpair v[RY0];
 #pragma unroll
     for (int k = 0; k < RY0; ++k) v[k] = p[k * (RY1 * S)];
@@ -336,13 +352,12 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
     }
   }
   // block sum without barriers of its own: the warps' sums to red[par] now, and warp 0 adds them after the
-  // barrier that the inverse stages need anyway -- at the end of the item, when no other warp waits for it,
-  // unless the block has its SM to itself (128^3: 9.63 against 9.82 ms at the end)
-  constexpr bool kLate = NT < 480;
+  // barrier that the inverse stages need anyway (the longer compensated sum at the end of the item, when no
+  // other warp waits for it)
+  constexpr bool kLate = PlaneSum<N>::compensated;
   PlaneSum<N>::warp(e_acc, red[par]);
   __syncthreads();
-  double* ep = epart + (long long)(c0 + cl) * N + y;
-  if (threadIdx.x < 32 && (!kLate || energy_only)) PlaneSum<N>::template block<NT / 32>(red[par], ep);
+  if (threadIdx.x < 32 && (!kLate || energy_only)) PlaneSum<N>::template block<NT / 32>(red[par], epart + (long long)(c0 + cl) * N + y);
   if (energy_only) return;
   // inverse z: elements e + 4 k of row x
 #pragma unroll 1
@@ -373,7 +388,7 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
 #pragma unroll
     for (int k = 0; k < R; ++k) dst[k * (4 * N)] = v[k];
   }
-  if (kLate && threadIdx.x < 32) PlaneSum<N>::template block<NT / 32>(red[par], ep);
+  if (kLate && threadIdx.x < 32) PlaneSum<N>::template block<NT / 32>(red[par], epart + (long long)(c0 + cl) * N + y);
 }
 
 template <int N, int NT, int MINB>
