@@ -1,4 +1,6 @@
-// Compile-time-geometry versions of the exchange passes for cubic grids of edge N.
+// Compile-time-geometry versions of the exchange passes for cubic grids of edge N.  The forward and x
+// passes here run the edges that are no multiple of 4 (50, 54, 90); the others have those of
+// hfx_ct_plane.cuh.
 //
 // Same algorithm and the same in-place DIF/DIT stage order as the runtime kernels in
 // hfx_kernels.cuh (so the digit-reversed storage order, and therefore the Coulomb table, are
@@ -78,7 +80,7 @@ __device__ __forceinline__ void stages(C* buf, const C* tw) {
 
 // forward stage 0 of column lines reading its input from global memory: line l's element e at
 // src[l + e*GES]; results go to buf[l*SLS + e*SES].  A barrier follows.  The loads go through L2
-// only (read once; in a persistent launch another block of the same launch may have written them).
+// only (read once).
 template <int R, int M, int LINES, int GES, int SLS, int SES, int N, int NT, typename C>
 __device__ __forceinline__ void stage_fwd_g2s(const C* __restrict__ src, C* __restrict__ buf,
                                               const C* __restrict__ twt) {
@@ -224,12 +226,8 @@ template <int N> struct PlaneSum {
 
 constexpr int kUnroll = 4;
 
-// threads per block of the compile-time plane kernels: 256, but 512 where the padded plane is so
-// large that one block fills an SM's shared memory (N = 128), so that 16 warps rather than 8 hide
-// the latency of each SM's single plane
-template <int N> struct PlaneThreads {
-  static constexpr int value = N * (N + 1) * 8 > 114 * 1024 ? 2 * kThreadsPlane : kThreadsPlane;
-};
+// threads per block of the one-stage-at-a-time plane kernels
+template <int N> struct PlaneThreads { static constexpr int value = kThreadsPlane; };
 
 // resident blocks per SM the plane kernels of edge N are built for: at most `cap`, and no more than
 // the padded plane (N (N+1) complex FP32 plus the twiddles, ~1 KB) lets fit in an SM's 228 KB of

@@ -282,8 +282,7 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
   constexpr int R = G::R, S = G::SX, PLANE = N * N;
   float2* wc = W + ((long long)cl * N + y) * PLANE;
   // forward x: elements j + 4 k of column z, straight from W; the loads go through L2 only (each is read
-  // once, and in a persistent launch another block of the same launch may have written it), and the
-  // first ones are issued before the barrier that ends the previous item's use of buf
+  // once), and the first ones are issued before the barrier that ends the previous item's use of buf
   if constexpr (NT > 4 * N) __syncthreads();
 #pragma unroll 1
   for (int id = threadIdx.x; id < 4 * N; id += NT) {

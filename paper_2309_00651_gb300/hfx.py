@@ -149,9 +149,17 @@ def _check(status: int) -> None:
         raise HFXError(status, msg.decode() if msg else "")
 
 
+# the current stream's handle without building a Stream object: a small SIN(R) update, launch and all,
+# 7.6 -> 4.7 us
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_handle(stream: Optional[torch.cuda.Stream]) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if stream is not None:
+        return int(stream.cuda_stream)
+    if _raw_stream is None:
+        return int(torch.cuda.current_stream().cuda_stream)
+    return int(_raw_stream(torch.cuda.current_device()))
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
