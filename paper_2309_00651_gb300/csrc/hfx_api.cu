@@ -377,6 +377,12 @@ static bool ragged_dense(const hfx_ctx* c) {
   return c->ct != nullptr && c->prec == HFX_PREC_FP32 && c->bsize == 8 && c->dense_tma && c->grid[0] % 4 == 0;
 }
 
+// whether the dense pass in use takes the ragged last block's pairs: the TMA form and the runtime-geometry
+// form do (27 orbitals on 54x60x72: call 1.33 -> 1.30 ms), the compile-time form with per-thread copies does not
+static bool ragged_rows(const hfx_ctx* c) {
+  return ragged_dense(c) || (dense_available(c) && !(c->ct && c->bsize == 8));
+}
+
 // Every device allocation the library makes for itself (context tables, schedules, batch tables)
 // goes through dev_alloc / dev_free: one place that counts what is held and that a test can make
 // fail (hfx_test_fail_allocation), so the error paths are exercised without exhausting a GPU.
@@ -750,7 +756,8 @@ constexpr size_t kGroupMin = size_t(64) << 20, kGroupMax = size_t(1) << 30;
 static Schedule make_host_schedule(const hfx_ctx* c, int n_orb) {
   Schedule S;
   build_schedule(S, n_orb, c->bsize, c->transform_budget, (size_t)c->N * cplx_size(c), dense_available(c),
-                 diag_available(c), ragged_dense(c));
+                 diag_available(c), ragged_rows(c));
+  S.dead_words = ragged_dense(c);
   const size_t per = (size_t)c->N * cplx_size(c);
   build_groups(S, c->ct && S.max_batch_couples * per >= kGroupMin ? (long long)(std::min(kGroupMax, c->transform_budget) / per) : 0);
   return S;
@@ -762,7 +769,7 @@ static bool two_buffers(const hfx_ctx* c, const Schedule& S) { return S.ngroups 
 // the couple table, then for the TMA dense pass (slots of at most 32 couples) one word per slot whose set
 // bits are the couples without pairs; both start as all ones
 static size_t couple_table_bytes(const Schedule& S) {
-  return (size_t)S.max_total_couples * sizeof(int4) + (S.ragged_rows ? (size_t)S.nslots * sizeof(unsigned) : 0);
+  return (size_t)S.max_total_couples * sizeof(int4) + (S.dead_words ? (size_t)S.nslots * sizeof(unsigned) : 0);
 }
 
 static Layout layout_of(const hfx_ctx* c, const Schedule& S, int n_orb, bool second_buffer) {
@@ -836,7 +843,8 @@ static hfx_status get_schedule(hfx_ctx* c, int n_orb, Schedule** out) {
 // every listed pair goes to its fixed place in the canonical couple layout of its block pair;
 // entries outside 0 <= i <= j < n_orb, and second copies of a pair, are flagged and skipped.
 // dead_words (the TMA dense pass: slots of at most 32 couples) loses the bit of every couple that gets
-// a pair, and off-diagonal pairs with the last, ragged block are laid out with its orbitals as rows
+// a pair; with ragged_rows, off-diagonal pairs with the last, ragged block are laid out with its orbitals
+// as rows
 struct PlaceArgs {
   const int2* pairs;
   long long P;
@@ -845,6 +853,7 @@ struct PlaceArgs {
   const int* slot_couple_base;
   int4* couples;
   unsigned* dead_words;
+  int ragged_rows;
   int* err;
 };
 __device__ __forceinline__ void place_pairs(const PlaceArgs& A, long long first, long long step) {
@@ -864,7 +873,7 @@ __device__ __forceinline__ void place_pairs(const PlaceArgs& A, long long first,
     const int si = min(bsize, n_orb - I0), sj = min(bsize, n_orb - J0);
     int t, c;
     if (bi != bj) {
-      t = dead_words && sj < bsize ? (j - J0) * bsize + (i - I0) : (i - I0) * sj + (j - J0);
+      t = A.ragged_rows && sj < bsize ? (j - J0) * bsize + (i - I0) : (i - I0) * sj + (j - J0);
       c = t >> 1;
     } else if (i != j) {
       const int a = i - I0, b = j - I0;  // a < b
@@ -1209,7 +1218,7 @@ static hfx_status run_passes(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
                         (const float2*)W, (const float2*)c->d_twct, (float*)vacc, vscale);
       else if (nd > 0)
         Passes<T>::y_acc_dense(g, dim3(nzc, g.n1, nd), dense_threads, smem_dense(c), st, S.b, orb, couples,
-                               S.d_dense_slots + S.dense_begin[b], S.d_slot_couple_base, S.d_slot_blocks, c0, W,
+                               S.d_dense_slots + S.dense_begin[b], S.d_slot_couple_base, S.d_slot_blocks, n_orb, c0, W,
                                (const C*)c->d_tw[1], vacc, vscale);
       if (nd > 0) close(kProfAcc, e0, st);
       const int ndg = S.diag_begin[b + 1] - S.diag_begin[b];
@@ -1282,7 +1291,7 @@ static hfx_status stage_call(hfx_ctx* c, Schedule& S, const Layout& L, const Cal
   float* dst = (float*)(ws + L.orb32);
   int4* couples = (int4*)(ws + L.couples);
   const PlaceArgs A{(const int2*)pairs, n_pairs, n_orb, S.b, S.nb, S.d_slot_of_bp, S.d_slot_couple_base, couples,
-                    S.ragged_rows ? (unsigned*)(couples + S.max_total_couples) : nullptr, c->d_err};
+                    S.dead_words ? (unsigned*)(couples + S.max_total_couples) : nullptr, S.ragged_rows ? 1 : 0, c->d_err};
   const bool place = n_pairs <= kPlaceHere;
   const int words = (int)(couple_table_bytes(S) / 4);
   const long long work = std::max<long long>(std::max(zero_bytes / 16, cast ? n / 4 : 0), place ? 1 : words);
@@ -1848,7 +1857,8 @@ extern "C" hfx_status hfx_apply_noalloc(hfx_ctx* c, const void* orbitals, int32_
     const size_t room = fixed < kNoallocScratchBytes ? kNoallocScratchBytes - fixed : 0;
     if (room >= (size_t)cap_max * couple_bytes + 256) {
       build_schedule(S, n_orb, c->bsize, room - 256, couple_bytes, dense_available(c), diag_available(c),
-                     ragged_dense(c));
+                     ragged_rows(c));
+      S.dead_words = ragged_dense(c);
       build_groups(S, 0);
       L = layout_of(c, S, n_orb, false);
     }

@@ -581,7 +581,7 @@ template <typename T, int B, int NP>
 __global__ void __launch_bounds__(DenseBounds<NP>::threads, DenseBounds<NP>::blocks)
 k_y_acc_dense(const __grid_constant__ Geo g, const T* __restrict__ orb, const int4* __restrict__ couples,
               const int* __restrict__ slot_list, const int* __restrict__ slot_couple_base,
-              const int2* __restrict__ slot_blocks, int c0, const cx<T>* __restrict__ W,
+              const int2* __restrict__ slot_blocks, int n_orb, int c0, const cx<T>* __restrict__ W,
               const cx<T>* __restrict__ tw2g, T* __restrict__ V, double vscale) {
   using C = cx<T>;
   constexpr int ZC = ZChunk<T>::value;
@@ -601,7 +601,10 @@ k_y_acc_dense(const __grid_constant__ Geo g, const T* __restrict__ orb, const in
   T* accI = phiI + B * pts;                    // [B][pts]
 
   const int2 blk = slot_blocks[slot];
-  const int I0 = blk.x * B, J0 = blk.y * B;
+  // a last block of fewer orbitals gives the rows (the staging lays its couples out that way)
+  const bool ragged = blk.y * B + B > n_orb;
+  const int I0 = (ragged ? blk.y : blk.x) * B, J0 = (ragged ? blk.x : blk.y) * B;
+  const int rows = min(B, n_orb - I0);
   const int cs = slot_couple_base[slot];
   const long long plane = (long long)n2 * n3;
   const long long rowoff = (long long)x * plane + z0;
@@ -609,7 +612,7 @@ k_y_acc_dense(const __grid_constant__ Geo g, const T* __restrict__ orb, const in
   // tiles of orbital row r -> ring buffer r % kDenseRing (empty couples and columns past n3 read as
   // zero); a row past the block commits an empty group so the group count stays uniform
   auto issue_row = [&](int r) {
-    if (r >= B) { cp_async_commit(); return; }
+    if (r >= rows) { cp_async_commit(); return; }
     C* dstb = tiles + (r % kDenseRing) * n2 * LN;
     for (int i = threadIdx.x; i < HB * n2 * (ZC / PER); i += blockDim.x) {
       const int v = i % (ZC / PER);
@@ -629,7 +632,7 @@ k_y_acc_dense(const __grid_constant__ Geo g, const T* __restrict__ orb, const in
   for (int i = threadIdx.x; i < B * pts; i += blockDim.x) {
     const int o = i / pts, p = i - o * pts;
     const int y = p / ZC, zz = p - y * ZC;
-    phiI[i] = zz < zcn ? __ldg(orb + (long long)(I0 + o) * g.N + rowoff + (long long)y * n3 + zz) : T(0);
+    phiI[i] = o < rows && zz < zcn ? __ldg(orb + (long long)(I0 + o) * g.N + rowoff + (long long)y * n3 + zz) : T(0);
   }
 
   // this thread's points
@@ -652,7 +655,7 @@ k_y_acc_dense(const __grid_constant__ Geo g, const T* __restrict__ orb, const in
   }
 
   const FastDiv ldiv = fastdiv_dev(LN);
-  for (int r = 0; r < B; ++r) {
+  for (int r = 0; r < rows; ++r) {
     issue_row(r + kDenseRing - 1);  // its buffer was last read in row r - 1 (barrier passed)
     cp_async_wait<kDenseRing - 1>();
     __syncthreads();  // row r's tiles (and the tables) visible to all threads
@@ -695,13 +698,14 @@ k_y_acc_dense(const __grid_constant__ Geo g, const T* __restrict__ orb, const in
 #pragma unroll
   for (int k = 0; k < NP; ++k)
 #pragma unroll
-    for (int j = 0; j < B; ++j) old[k][j] = ok[k] ? __ldcg(V + (long long)(I0 + j) * g.N + goff[k]) : T(0);
+    for (int j = 0; j < B; ++j) old[k][j] = ok[k] && j < rows ? __ldcg(V + (long long)(I0 + j) * g.N + goff[k]) : T(0);
 #pragma unroll
   for (int k = 0; k < NP; ++k) {
     if (!ok[k]) continue;
     const int p = pp[k];
 #pragma unroll
-    for (int j = 0; j < B; ++j) V[(long long)(I0 + j) * g.N + goff[k]] = old[k][j] + vs * accI[j * pts + p];
+    for (int j = 0; j < B; ++j)
+      if (j < rows) V[(long long)(I0 + j) * g.N + goff[k]] = old[k][j] + vs * accI[j * pts + p];
   }
 }
 

@@ -53,13 +53,13 @@ void Passes<Real>::x_coulomb(const Geo& g, int grid, size_t smem, cudaStream_t s
 template <>
 void Passes<Real>::y_acc_dense(const Geo& g, dim3 grid, int threads, size_t smem, cudaStream_t st, int b,
                                const Real* orb, const int4* couples, const int* slot_list, const int* slot_couple_base,
-                               const int2* slot_blocks, int c0, const cx<Real>* W, const cx<Real>* tw2, Real* V,
+                               const int2* slot_blocks, int n_orb, int c0, const cx<Real>* W, const cx<Real>* tw2, Real* V,
                                double vscale) {
   // points per thread so that one block of at most kDenseMaxThreads threads covers the tile
   const int pts = g.n2 * ZChunk<Real>::value;
   const bool np4 = pts > 2 * DenseBounds<2>::threads;
 #define HFX_DENSE(BB, NPP)                                                                                      \
-  k_y_acc_dense<Real, BB, NPP><<<grid, threads, smem, st>>>(g, orb, couples, slot_list, slot_couple_base, slot_blocks, \
+  k_y_acc_dense<Real, BB, NPP><<<grid, threads, smem, st>>>(g, orb, couples, slot_list, slot_couple_base, slot_blocks, n_orb, \
                                                             c0, W, tw2, V, vscale)
   if (b == 8) { if (np4) HFX_DENSE(8, 4); else HFX_DENSE(8, 2); }
   else { if (np4) HFX_DENSE(4, 4); else HFX_DENSE(4, 2); }

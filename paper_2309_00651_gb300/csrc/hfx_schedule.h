@@ -27,6 +27,7 @@ struct Schedule {
   std::vector<int> dense_slots, generic_slots, diag_slots;  // concatenated over batches
   std::vector<int> dense_begin, generic_begin, diag_begin;  // [nbatches + 1] offsets into the lists
   bool ragged_rows = false;             // layout of ragged off-diagonal block pairs (build_schedule)
+  bool dead_words = false;              // the couple table has a word per slot (the TMA dense pass)
   // consecutive batches whose forward and x passes run as one launch each (build_groups): group q is
   // batches group_begin[q] .. group_begin[q + 1] - 1
   std::vector<int> group_begin;
