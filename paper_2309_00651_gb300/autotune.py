@@ -105,8 +105,8 @@ BATCH_BUDGETS = (1 << 30, 512 << 20, 256 << 20, 2 << 30)
 
 def tune_batch(exchanges, run_persistent, run_sequential, n_orbs, n_pairs,
                budgets: Iterable[int] = BATCH_BUDGETS, steps: int = 2, timer=None) -> dict:
-    """Pick the pair-batch size (per-context transform budget) of the uneven batch's persistent
-    launch, then keep the persistent form or the one-call-per-problem form, whichever is faster.
+    """Pick the pair-batch size (per-context transform budget) of the uneven batch's batched
+    call ("persistent"), then keep it or the one-call-per-problem form, whichever is faster.
 
     exchanges: the Exchange of every problem; run_persistent / run_sequential: callables that
     run the whole batch once in that form; n_orbs, n_pairs: per problem (for the workspaces).

@@ -219,7 +219,8 @@ def _batch_args(ctxs, args):
 
 
 def hfx_apply_batched(ctxs, args, stream: Optional[torch.cuda.Stream] = None) -> None:
-    """All problems in one persistent launch.  ctxs: list of contexts; args: list of
+    """All problems share the GPU: small ones in one persistent launch, others forked onto their
+    contexts' own streams and joined.  ctxs: list of contexts; args: list of
     (orbitals, pairs, ex, vxphi, flags)."""
     n, carr, aarr = _batch_args(ctxs, args)
     _check(load_library().hfx_apply_batched(carr, aarr, n, _stream_handle(stream)))
