@@ -196,31 +196,28 @@ __device__ __forceinline__ void two_sum(float& s, float& e, float a, float ea) {
   s = t;
 }
 
-// Sum of one value per thread over a block for the plane energies: a tree per warp into red, then one over
-// the warps.  FP32 trees for the edges where that was measured to be enough (E within 2e-7); the others,
-// whose planes the runtime-geometry pass sums in FP64, carry the rounding errors along (about 48 bits),
-// which costs the x pass 1 to 3%.
-template <int N> struct PlaneSum {
-  static constexpr bool compensated = !(N == 32 || N == 48 || N == 64 || N == 72 || N == 80 || N == 90 || N == 96 || N == 128);
-  static __device__ __forceinline__ void warp(float s, float2* red) {
-    float e = 0.f;
+// A plane's energy: each thread adds its FP32 partials, one per butterfly, with their rounding errors carried
+// along, then a tree per warp into red and one over the warps do the same (about 48 bits).  So the only FP32
+// roundings are those inside a butterfly, as in the runtime-geometry pass, whose other sums are FP64.  Those
+// would take the narrow FP64 pipe here; plain FP32 sums were up to 2e-8 off (64^3, F = 1 everywhere:
+// 9e-9 rms over eight cells, now 1e-9).  Against those the x pass takes up to 1% more, 1.8% at 80^3
+// (64 orbitals, us a call, plain / this: 64^3 857 / 866, 72^3 1373 / 1387, 80^3 1882 / 1914, 96^3 3904 / 3950,
+// 128^3, 32 orbitals, 2746 / 2772).
+struct PlaneSum {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float a) { two_sum(s, e, a, 0.f); }
+  __device__ __forceinline__ void warp(float2* red) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      if constexpr (compensated) two_sum(s, e, __shfl_down_sync(0xffffffffu, s, o), __shfl_down_sync(0xffffffffu, e, o));
-      else s += __shfl_down_sync(0xffffffffu, s, o);
-    }
+    for (int o = 16; o > 0; o >>= 1) two_sum(s, e, __shfl_down_sync(0xffffffffu, s, o), __shfl_down_sync(0xffffffffu, e, o));
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_float2(s, e);
   }
   // by the threads of warp 0
   template <int NW> static __device__ __forceinline__ void block(const float2* red, double* out) {
     float2 r = threadIdx.x < NW ? red[threadIdx.x] : make_float2(0.f, 0.f);
 #pragma unroll
-    for (int o = NW > 16 ? 16 : NW > 8 ? 8 : NW > 4 ? 4 : NW > 2 ? 2 : 1; o > 0; o >>= 1) {
-      if constexpr (compensated)
-        two_sum(r.x, r.y, __shfl_down_sync(0xffffffffu, r.x, o), __shfl_down_sync(0xffffffffu, r.y, o));
-      else r.x += __shfl_down_sync(0xffffffffu, r.x, o);
-    }
-    if (threadIdx.x == 0) *out = compensated ? widen_exact(r.x) + widen_exact(r.y) : widen_exact(r.x);
+    for (int o = NW > 16 ? 16 : NW > 8 ? 8 : NW > 4 ? 4 : NW > 2 ? 2 : 1; o > 0; o >>= 1)
+      two_sum(r.x, r.y, __shfl_down_sync(0xffffffffu, r.x, o), __shfl_down_sync(0xffffffffu, r.y, o));
+    if (threadIdx.x == 0) *out = widen_exact(r.x) + widen_exact(r.y);
   }
 };
 
@@ -356,9 +353,8 @@ __device__ __forceinline__ void x_coulomb_ct_item(const int4* __restrict__ coupl
   stage_fwd_g2s<P.r[0], P.m[0], N, PLANE, 1, S, N, NT>(wc, buf, tw + P.twoff[0]);
   stages<N, false, 1, P.ns - 1, N, 1, S, NT>(buf, tw);  // remaining x stages but the last
   // last forward x stage (no twiddles) + Coulomb + energy + first inverse x stage
-  // the plane's energy partial in FP32 (a few terms per thread, then a tree over the block),
-  // widened once; the partials of all planes and couples are summed in FP64
-  T e_acc = T(0);
+  // the plane's energy: FP32 within a butterfly, then PlaneSum; the planes and couples are summed in FP64
+  PlaneSum energy;
   {
     constexpr int TOTAL = N * (N / RL);
     const T* vy = vtab + (long long)y * N;
@@ -380,7 +376,7 @@ __device__ __forceinline__ void x_coulomb_ct_item(const int4* __restrict__ coupl
         v[k].x *= vg[k];
         v[k].y *= vg[k];
       }
-      e_acc += e;
+      energy.add(e);
       if (!energy_only) {
         Dft<RL, 1, C>::run(v);
 #pragma unroll
@@ -391,9 +387,9 @@ __device__ __forceinline__ void x_coulomb_ct_item(const int4* __restrict__ coupl
   static_assert(sizeof(T) == 4, "compile-time passes are FP32");
   // block sum without barriers of its own: the warps' sums to red[par] now, and warp 0 adds them after the
   // barrier that the inverse stages need anyway
-  PlaneSum<N>::warp(e_acc, red[par]);
+  energy.warp(red[par]);
   __syncthreads();
-  if (threadIdx.x < 32) PlaneSum<N>::template block<(NT + 31) / 32>(red[par], epart + (long long)(c0 + cl) * N + y);
+  if (threadIdx.x < 32) PlaneSum::block<(NT + 31) / 32>(red[par], epart + (long long)(c0 + cl) * N + y);
   if (energy_only) return;
   // inverse transforms along different axes commute: z first (rows), then the remaining x
   // stages, the last of which writes W directly

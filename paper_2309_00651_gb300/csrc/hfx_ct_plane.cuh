@@ -299,9 +299,9 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
     for (int k = 0; k < R; ++k) p[G::place(k) * (4 * S) + 2 * ((G::place(k) >> 1) & 1)] = v[k];
   }
   // the tile x = 4 X .. 4 X + 3, z = 4 Z .. 4 Z + 3: last forward x stage, v(G) and the energy, first
-  // inverse x stage, first inverse z stage.  The plane's energy: a few tiles' terms per thread in FP32,
-  // then PlaneSum over the block; planes and couples are summed in FP64
-  float e_acc = 0.f;
+  // inverse x stage, first inverse z stage.  The plane's energy: FP32 within a butterfly, then PlaneSum;
+  // planes and couples are summed in FP64
+  PlaneSum energy;
   const float* vy = vtab + (long long)y * N;
   __syncthreads();
 #pragma unroll 1
@@ -325,9 +325,9 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
       v[2][f] = cpair{b.x, b.y};
       v[3][f] = cpair{b.z, b.w};
     }
-    float en = 0.f;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
+      float en = 0.f;
       Dft<4, -1, cpair>::run(v[e]);
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
@@ -336,8 +336,8 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
         v[e][f].x *= vg;
         v[e][f].y *= vg;
       }
+      energy.add(en);
     }
-    e_acc += en;
     if (!energy_only) {
 #pragma unroll
       for (int e = 0; e < 4; ++e) Dft<4, 1, cpair>::run(v[e]);
@@ -351,12 +351,11 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
     }
   }
   // block sum without barriers of its own: the warps' sums to red[par] now, and warp 0 adds them after the
-  // barrier that the inverse stages need anyway (the longer compensated sum at the end of the item, when no
-  // other warp waits for it)
-  constexpr bool kLate = PlaneSum<N>::compensated;
-  PlaneSum<N>::warp(e_acc, red[par]);
+  // barrier that the inverse stages need anyway (at the end of the item instead it cost the x pass 2% more where
+  // one or two planes fit an SM)
+  energy.warp(red[par]);
   __syncthreads();
-  if (threadIdx.x < 32 && (!kLate || energy_only)) PlaneSum<N>::template block<NT / 32>(red[par], epart + (long long)(c0 + cl) * N + y);
+  if (threadIdx.x < 32) PlaneSum::block<NT / 32>(red[par], epart + (long long)(c0 + cl) * N + y);
   if (energy_only) return;
   // inverse z: elements e + 4 k of row x
 #pragma unroll 1
@@ -387,7 +386,6 @@ __device__ __forceinline__ void x_plane_item(int c0, float2* __restrict__ W, con
 #pragma unroll
     for (int k = 0; k < R; ++k) dst[k * (4 * N)] = v[k];
   }
-  if (kLate && threadIdx.x < 32) PlaneSum<N>::template block<NT / 32>(red[par], epart + (long long)(c0 + cl) * N + y);
 }
 
 template <int N, int NT, int MINB>
