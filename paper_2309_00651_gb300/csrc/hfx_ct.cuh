@@ -178,13 +178,15 @@ __device__ __forceinline__ void ld2(const double2* src, double2& a, double2& b) 
 }
 
 // FP32 -> FP64, exact for normal numbers and +-0, with integer operations only (sign, exponent
-// rebias 127 -> 1023, fraction widened); FP32 subnormals flush to zero.  The flushes below use it
-// so that their only FP64 instruction is the final add (the FP64 pipe of this part is narrow).
+// rebias 127 -> 1023, fraction widened); infinities and NaNs stay what they are, FP32 subnormals flush to
+// zero.  The flushes below use it so that their only FP64 instruction is the final add (the FP64 pipe of
+// this part is narrow).
 __device__ __forceinline__ double widen_exact(float v) {
   const unsigned u = __float_as_uint(v);
   const unsigned mag = u & 0x7fffffffu, sign = u & 0x80000000u;
   const bool tiny = mag < 0x00800000u;
-  const unsigned hi = tiny ? sign : (((mag >> 3) + 0x38000000u) | sign);
+  const unsigned top = (mag >> 3) + 0x38000000u;
+  const unsigned hi = tiny ? sign : ((mag >= 0x7f800000u ? top | 0x7ff00000u : top) | sign);
   const unsigned lo = tiny ? 0u : (mag << 29);
   return __hiloint2double((int)hi, (int)lo);
 }
@@ -217,7 +219,8 @@ struct PlaneSum {
 #pragma unroll
     for (int o = NW > 16 ? 16 : NW > 8 ? 8 : NW > 4 ? 4 : NW > 2 ? 2 : 1; o > 0; o >>= 1)
       two_sum(r.x, r.y, __shfl_down_sync(0xffffffffu, r.x, o), __shfl_down_sync(0xffffffffu, r.y, o));
-    if (threadIdx.x == 0) *out = widen_exact(r.x) + widen_exact(r.y);
+    // (a sum that is not finite has no rounding errors to add)
+    if (threadIdx.x == 0) *out = widen_exact(r.x) + (r.x - r.x == 0.f ? widen_exact(r.y) : 0.0);
   }
 };
 
