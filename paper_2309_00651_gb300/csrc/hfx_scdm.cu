@@ -179,7 +179,6 @@ __global__ void __launch_bounds__(kPickThreads, 1) k_scdm_pick(const double* __r
   const T* Q = QS ? qs : qt;
   // q_0 .. q_{j-1} are there (the update before this kernel let it start after its own wait for them); the
   // maxima and the residual norms are not
-  cudaTriggerProgrammaticLaunchCompletion();
   if (QS && j > 0) {
     constexpr int EPC = 16 / (int)sizeof(T);
     const int cpr = (j + EPC - 1) / EPC;
@@ -276,6 +275,11 @@ __global__ void __launch_bounds__(kPickThreads, 1) k_scdm_pick(const double* __r
     }
     __syncthreads();
   }
+  // The update may start: only now, because its blocks fill every SM and wait there for this kernel's end.
+  // Started with the pick they took the SMs from other streams (8 calls of 48 orbitals on 48^3 beside a
+  // localisation of 128 on 72^3: 9.7 ms, now 8.3; alone 5.4) and from the update before, and slowed the pick:
+  // 128 orbitals on 72^3 5.88 -> 5.70 ms, 63 2.86 -> 2.13, 40 on 80^3 1.58 -> 1.33.
+  cudaTriggerProgrammaticLaunchCompletion();
   const double ss = threadIdx.x < n ? (double)a[threadIdx.x] * (double)a[threadIdx.x] : 0.0;
   const double rn2 = sum_first_n(ss, n, red);
   if (threadIdx.x == 0) {
