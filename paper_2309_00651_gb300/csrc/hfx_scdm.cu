@@ -299,6 +299,27 @@ __global__ void __launch_bounds__(kPickThreads, 1) k_scdm_pick(const double* __r
   }
 }
 
+// c_k += sum_u q[u] row[u N + k kUpdThreads] over `rows` rows (all R of them with FULL, else fewer than R: a
+// test that is the same for every thread), all of whose loads are in flight together
+template <typename T, int R, bool FULL>
+__device__ __forceinline__ void dot_rows(const T* q, const T* __restrict__ row, long long N, int rows,
+                                         const bool (&in)[UpdShape<T>::points], T (&c)[UpdShape<T>::points]) {
+  constexpr int kPts = UpdShape<T>::points;
+  T v[R][kPts];
+#pragma unroll
+  for (int u = 0; u < R; ++u)
+    if (FULL || u < rows) {
+#pragma unroll
+      for (int k = 0; k < kPts; ++k) v[u][k] = in[k] ? row[(long long)u * N + k * kUpdThreads] : T(0);
+    }
+#pragma unroll
+  for (int u = 0; u < R; ++u)
+    if (FULL || u < rows) {
+#pragma unroll
+      for (int k = 0; k < kPts; ++k) c[k] = fma(q[u], v[u][k], c[k]);
+    }
+}
+
 // step j: c_p = q_j . Psi^T[:, p], nu_p -= c_p^2 (picked points stay at -1), per-block maxima; UpdShape
 // points per thread and rows in flight.
 //
@@ -306,10 +327,13 @@ __global__ void __launch_bounds__(kPickThreads, 1) k_scdm_pick(const double* __r
 // bandwidth bounds it.  Psi exceeds L2 but not by much, and an even step takes its runs of grid points
 // (`run` of them per block and round) from first to last, an odd one from last to first: each step begins
 // with what the one before left in L2; the dot products and the picks do not depend on the order of the
-// points.  A round is a chain of n / rows load latencies, so few rounds and many rows in flight win:
-// 128 orbitals on 72^3, whole localisation, 4 points a thread and no order 7.79 ms; 4 rounds with 16, 32,
-// 64 rows 7.25, 6.72, 5.93; 6 and 8 rounds lose.  The launches overlap (see launch_overlapped): 48 orbitals
-// on 48^3, which fits L2, 1.25 -> 1.04 ms, 20 on 32^3 0.40 -> 0.33.
+// points.  A round is a chain of load latencies, one for every `rows` rows and one for each group of what is
+// left, so few rounds and many rows in flight win: 128 orbitals on 72^3, whole localisation, 4 points a thread
+// and no order 7.79 ms; 4 rounds with 16, 32, 64 rows 7.25, 6.72, 5.93; 6 and 8 rounds lose.  What is left
+// eight at a time, as before / in these groups, ms: 63 on 72^3 2.13 / 1.83, 127 on 72^3 7.01 / 5.85, 127 on
+// 80^3 9.35 / 7.46, 20 on 48^3 0.428 / 0.409 (all of it in one tested group of 64 spills; one of 32 made 20 on
+// 72^3 0.63 instead of 0.54).  The launches overlap (see launch_overlapped): 48 orbitals on 48^3, which fits
+// L2, 1.26 -> 0.99 ms with the groups, 20 on 32^3 0.40 -> 0.34.
 template <typename T>
 __global__ void __launch_bounds__(kUpdThreads, kUpdBlocksPerSm) k_scdm_update(const T* __restrict__ A, long long N, int n,
                                                              const T* __restrict__ qt, long long ldt, int j, int run,
@@ -344,22 +368,21 @@ __global__ void __launch_bounds__(kUpdThreads, kUpdBlocksPerSm) k_scdm_update(co
     if (!in[0]) continue;
     const T* row = A + p0;
     int i = 0;
-    for (; i + kRows <= n; i += kRows) {
-      T v[kRows][kPts];
-#pragma unroll
-      for (int u = 0; u < kRows; ++u)
-#pragma unroll
-        for (int k = 0; k < kPts; ++k) v[u][k] = in[k] ? row[(long long)(i + u) * N + k * kUpdThreads] : T(0);
-#pragma unroll
-      for (int u = 0; u < kRows; ++u)
-#pragma unroll
-        for (int k = 0; k < kPts; ++k) c[k] = fma(q[i + u], v[u][k], c[k]);
+    for (; i + kRows <= n; i += kRows) dot_rows<T, kRows, true>(q + i, row + (long long)i * N, N, kRows, in, c);
+    // what is left: half as many rows, a quarter and an eighth, then fewer than that
+    if (i + kRows / 2 <= n) {
+      dot_rows<T, kRows / 2, true>(q + i, row + (long long)i * N, N, kRows / 2, in, c);
+      i += kRows / 2;
     }
-#pragma unroll 8
-    for (; i < n; ++i)
-#pragma unroll
-      for (int k = 0; k < kPts; ++k)
-        if (in[k]) c[k] = fma(q[i], row[(long long)i * N + k * kUpdThreads], c[k]);
+    if (i + kRows / 4 <= n) {
+      dot_rows<T, kRows / 4, true>(q + i, row + (long long)i * N, N, kRows / 4, in, c);
+      i += kRows / 4;
+    }
+    if (i + kRows / 8 <= n) {
+      dot_rows<T, kRows / 8, true>(q + i, row + (long long)i * N, N, kRows / 8, in, c);
+      i += kRows / 8;
+    }
+    if (i < n) dot_rows<T, kRows / 8, false>(q + i, row + (long long)i * N, N, n - i, in, c);
 #pragma unroll
     for (int k = 0; k < kPts; ++k) {
       if (!in[k]) continue;
