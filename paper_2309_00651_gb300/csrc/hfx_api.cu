@@ -207,6 +207,7 @@ struct hfx_ctx {
   void* d_dftb = nullptr;
   int blocks_fwd_tc = 1;
   std::map<int, std::unique_ptr<Schedule>> sched;  // by n_orb
+  mutable std::mutex sched_mu;  // hfx_workspace_bytes may run beside a call that adds to sched
   // queue tables of hfx_apply_batched when this context comes first in a batch
   void* d_batch = nullptr;
   size_t batch_bytes = 0;
@@ -801,13 +802,17 @@ static Layout layout_of(const hfx_ctx* c, const Schedule& S, int n_orb, bool sec
 extern "C" size_t hfx_workspace_bytes(const hfx_ctx* c, int32_t n_orb, int64_t n_pairs) {
   if (!c || n_orb <= 0 || n_pairs < 0) return 0;
   (void)n_pairs;
-  const auto it = c->sched.find(n_orb);  // (dropped when a setting that it depends on changes)
-  if (it != c->sched.end()) return layout_of(c, *it->second, n_orb, two_buffers(c, *it->second)).total;
+  {
+    std::lock_guard<std::mutex> lk(c->sched_mu);
+    const auto it = c->sched.find(n_orb);  // (dropped when a setting that it depends on changes)
+    if (it != c->sched.end()) return layout_of(c, *it->second, n_orb, two_buffers(c, *it->second)).total;
+  }
   const Schedule S = make_host_schedule(c, n_orb);
   return layout_of(c, S, n_orb, two_buffers(c, S)).total;
 }
 
 static hfx_status get_schedule(hfx_ctx* c, int n_orb, Schedule** out) {
+  std::lock_guard<std::mutex> lk(c->sched_mu);
   auto it = c->sched.find(n_orb);
   if (it != c->sched.end()) { *out = it->second.get(); return HFX_OK; }
   std::unique_ptr<Schedule> S(new Schedule(make_host_schedule(c, n_orb)));
@@ -1910,6 +1915,7 @@ extern "C" hfx_status hfx_set_tuning(hfx_ctx* c, int32_t block, size_t batch_byt
   c->pipeline = pipeline != 0;
   // cached schedules depend on the block size and the budget: drop them (device tables freed after
   // the device is idle, since a call in flight may still read them)
+  std::lock_guard<std::mutex> lk(c->sched_mu);
   if (!c->sched.empty()) {
     cudaDeviceSynchronize();
     for (auto& kv : c->sched) {
