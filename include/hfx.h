@@ -120,6 +120,15 @@ hfx_status hfx_create(const hfx_box* box, const int32_t grid[3], double ecut, hf
  * (Library plumbing; the paper has no counterpart.) */
 size_t hfx_workspace_bytes(const hfx_ctx* c, int32_t n_orb, int64_t n_pairs);
 
+/* hfx_workspace_bytes_least -- the least workspace that hfx_apply accepts, for a device without room for
+ * hfx_workspace_bytes: batches of at most 1 GiB of transforms (of batch_bytes after hfx_set_tuning), each with
+ * launches of its own (the first such call for an n_orb uploads its schedule table, as the first call of all
+ * does).  A call takes what the workspace holds; results do not depend on it beyond rounding
+ * order, times do: 256 orbitals on 96^3 take 138 ms in 5.9 GB and 144 to 149 in 3.9 GB, 64 on 64^3 2.4 ms
+ * in 2.3 GB and 2.5 to 2.6 in 0.74 GB.  Returns 0 on bad arguments.
+ * (Library plumbing; the paper has no counterpart.) */
+size_t hfx_workspace_bytes_least(const hfx_ctx* c, int32_t n_orb, int64_t n_pairs);
+
 /* hfx_set_workspace -- hand the context a caller-owned device buffer (e.g. a torch tensor)
  * of `bytes` bytes, 256-byte aligned.  The context keeps the pointer until it is replaced
  * or the context is destroyed; it never frees it.  Calls that use the same context must
@@ -139,7 +148,8 @@ hfx_status hfx_set_workspace(hfx_ctx* c, void* dev_ptr, size_t bytes);
  *   vxphi    : device FP64 [n_orb][n1][n2][n3] receiving V_x phi; NULL only with
  *              HFX_ENERGY_ONLY.
  *   cuda_stream : stream to enqueue on.
- * Needs a workspace of at least hfx_workspace_bytes(c, n_orb, n_pairs).  Asynchronous:
+ * Needs a workspace of hfx_workspace_bytes(c, n_orb, n_pairs), or at least of
+ * hfx_workspace_bytes_least (in smaller batches).  Asynchronous:
  * results are valid once the stream reaches them.  Deterministic: the same inputs give
  * bit-identical results. */
 hfx_status hfx_apply(hfx_ctx* c, const void* orbitals, int32_t n_orb, const int32_t* pairs,
@@ -176,7 +186,7 @@ typedef struct {
  *   Rules: same argument rules per problem as hfx_apply; one distinct context per problem; every
  *   context needs the same precision and device and planes that fit in shared memory
  *   (HFX_ERR_UNSUPPORTED_GRID otherwise); each context's workspace must hold hfx_workspace_bytes
- *   for its problem; batched calls led by one context must not overlap on the GPU.  The queue tables
+ *   (or hfx_workspace_bytes_least) for its problem; batched calls led by one context must not overlap on the GPU.  The queue tables
  *   (sized by either form) live in a device buffer owned by the first context (ctxs[0]); the first call that needs a larger one
  *   allocates it (and synchronises the stream), so make that call before any stream capture --
  *   during capture such a call is rejected with HFX_ERR_INVALID_ARG.  Stops at the first problem

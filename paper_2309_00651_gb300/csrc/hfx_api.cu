@@ -179,6 +179,9 @@ struct hfx_ctx {
   // orbitals on 96^3 took 150.3, 145.2, 137.6 and 135.5 ms with 0.5, 1, 2 and 4 GiB, 64 on 128^3 29.0, 27.4,
   // 26.3 and 26.3; rounds that fit 1 GiB (72^3) do not change
   size_t transform_budget = size_t(2) << 30;
+  // the same for a workspace that does not hold such batches (hfx_workspace_bytes_least); what the caller sets
+  // is for both
+  size_t lean_budget = size_t(1) << 30;
   int blocks_fwd = 1, blocks_x = 1;
   int gen_grp = 1, gen_phi = 0;  // generic accumulate pass: couples per group, orbital tiles on chip
   // second stream and events: the forward and x passes of batch b+1 run beside the accumulate
@@ -206,7 +209,7 @@ struct hfx_ctx {
   bool tc_dft = false;
   void* d_dftb = nullptr;
   int blocks_fwd_tc = 1;
-  std::map<int, std::unique_ptr<Schedule>> sched;  // by n_orb
+  std::map<std::pair<int, bool>, std::unique_ptr<Schedule>> sched;  // by n_orb and whether it is the lean one
   mutable std::mutex sched_mu;  // hfx_workspace_bytes may run beside a call that adds to sched
   // queue tables of hfx_apply_batched when this context comes first in a batch
   void* d_batch = nullptr;
@@ -622,7 +625,7 @@ extern "C" hfx_status hfx_create(const hfx_box* box, const int32_t grid[3], doub
   c->alpha = alpha;
   c->prec = prec;
   if (const char* s = std::getenv("HFX_BLOCK")) c->bsize = std::max(1, std::min(32, atoi(s)));
-  if (const char* s = std::getenv("HFX_BATCH_MB")) c->transform_budget = (size_t)std::max(1, atoi(s)) << 20;
+  if (const char* s = std::getenv("HFX_BATCH_MB")) c->transform_budget = c->lean_budget = (size_t)std::max(1, atoi(s)) << 20;
   if (const char* s = std::getenv("HFX_PIPELINE")) c->pipeline = atoi(s) != 0;
   if (const char* s = std::getenv("HFX_NO_TC")) c->ace_tc = atoi(s) == 0;
   if (const char* s = std::getenv("HFX_DENSE_TMA")) c->dense_tma = atoi(s) != 0;
@@ -754,13 +757,13 @@ static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 // 666; together lost at 48^3 with 24 (201 / 221) and 32^3 with 64 (371 / 409), whose batches are 44 and 33 MB.
 constexpr size_t kGroupMin = size_t(64) << 20, kGroupMax = size_t(1) << 30;
 
-static Schedule make_host_schedule(const hfx_ctx* c, int n_orb) {
+// lean: batches of at most lean_budget, a launch each, for a workspace that does not hold the others
+static Schedule make_host_schedule(const hfx_ctx* c, int n_orb, bool lean = false) {
   Schedule S;
-  build_schedule(S, n_orb, c->bsize, c->transform_budget, (size_t)c->N * cplx_size(c), dense_available(c),
-                 diag_available(c), ragged_rows(c));
+  const size_t per = (size_t)c->N * cplx_size(c), budget = lean ? c->lean_budget : c->transform_budget;
+  build_schedule(S, n_orb, c->bsize, budget, per, dense_available(c), diag_available(c), ragged_rows(c));
   S.dead_words = ragged_dense(c);
-  const size_t per = (size_t)c->N * cplx_size(c);
-  build_groups(S, c->ct && S.max_batch_couples * per >= kGroupMin ? (long long)(std::min(kGroupMax, c->transform_budget) / per) : 0);
+  build_groups(S, !lean && c->ct && S.max_batch_couples * per >= kGroupMin ? (long long)(std::min(kGroupMax, budget) / per) : 0);
   return S;
 }
 
@@ -799,23 +802,44 @@ static Layout layout_of(const hfx_ctx* c, const Schedule& S, int n_orb, bool sec
   return L;
 }
 
+// f of n_orb's schedule: the context's where it has one (dropped when a setting that it depends on changes)
+template <typename F>
+static size_t with_schedule(const hfx_ctx* c, int n_orb, bool lean, F f) {
+  {
+    std::lock_guard<std::mutex> lk(c->sched_mu);
+    const auto it = c->sched.find({n_orb, lean});
+    if (it != c->sched.end()) return f(*it->second);
+  }
+  return f(make_host_schedule(c, n_orb, lean));
+}
+
 extern "C" size_t hfx_workspace_bytes(const hfx_ctx* c, int32_t n_orb, int64_t n_pairs) {
   if (!c || n_orb <= 0 || n_pairs < 0) return 0;
   (void)n_pairs;
-  {
-    std::lock_guard<std::mutex> lk(c->sched_mu);
-    const auto it = c->sched.find(n_orb);  // (dropped when a setting that it depends on changes)
-    if (it != c->sched.end()) return layout_of(c, *it->second, n_orb, two_buffers(c, *it->second)).total;
-  }
-  const Schedule S = make_host_schedule(c, n_orb);
-  return layout_of(c, S, n_orb, two_buffers(c, S)).total;
+  return with_schedule(c, n_orb, false, [&](const Schedule& S) { return layout_of(c, S, n_orb, two_buffers(c, S)).total; });
 }
 
-static hfx_status get_schedule(hfx_ctx* c, int n_orb, Schedule** out) {
+// the least a call accepts (pipelined: hfx_apply, else a batched call's problem): the lean schedule's layout.
+// Where that has two buffers, the words of the TMA dense pass need not fit beside them: the call then runs
+// with one.
+static size_t least_bytes(const hfx_ctx* c, int32_t n_orb, bool pipelined) {
+  return with_schedule(c, n_orb, true, [&](const Schedule& S) {
+    const bool two = pipelined && two_buffers(c, S);
+    const size_t words = align256(couple_table_bytes(S)) - align256((size_t)S.max_total_couples * sizeof(int4));
+    return layout_of(c, S, n_orb, two).total - (two ? words : 0);
+  });
+}
+
+extern "C" size_t hfx_workspace_bytes_least(const hfx_ctx* c, int32_t n_orb, int64_t n_pairs) {
+  if (!c || n_orb <= 0 || n_pairs < 0) return 0;
+  return std::min(least_bytes(c, n_orb, true), hfx_workspace_bytes(c, n_orb, n_pairs));
+}
+
+static hfx_status get_schedule(hfx_ctx* c, int n_orb, bool lean, Schedule** out) {
   std::lock_guard<std::mutex> lk(c->sched_mu);
-  auto it = c->sched.find(n_orb);
+  auto it = c->sched.find({n_orb, lean});
   if (it != c->sched.end()) { *out = it->second.get(); return HFX_OK; }
-  std::unique_ptr<Schedule> S(new Schedule(make_host_schedule(c, n_orb)));
+  std::unique_ptr<Schedule> S(new Schedule(make_host_schedule(c, n_orb, lean)));
   auto up = [&](void** dst, const void* src, size_t bytes) -> hfx_status {
     if (bytes == 0) {  // an empty list still gets a valid (unused) device pointer
       cudaError_t e = dev_alloc(dst, 16);
@@ -838,8 +862,33 @@ static hfx_status get_schedule(hfx_ctx* c, int n_orb, Schedule** out) {
     return st;
   }
   *out = S.get();
-  c->sched[n_orb] = std::move(S);
+  c->sched[{n_orb, lean}] = std::move(S);
   return HFX_OK;
+}
+
+// The schedule and layout of a call in the context's workspace: what hfx_workspace_bytes asks for where it
+// fits, else the lean schedule, with a second buffer (*two) or without.  ms in the first, the second and the
+// third: 64 orbitals on 64^3 2.39 (2.3 GB), 2.51 and 2.63 (0.74 GB); 256 on 96^3 138.5 (5.9 GB), 143.6 and 148.6
+// (3.9 GB).
+static hfx_status fit_workspace(hfx_ctx* c, int n_orb, bool pipelined, Schedule** S, Layout* L, bool* two) {
+  hfx_status s = get_schedule(c, n_orb, false, S);
+  if (s != HFX_OK) return s;
+  *two = pipelined && two_buffers(c, **S);
+  *L = layout_of(c, **S, n_orb, *two);
+  if (c->ws && c->ws_bytes >= L->total) return HFX_OK;
+  const size_t need = L->total;
+  if (c->ws && c->ws_bytes >= least_bytes(c, n_orb, pipelined)) {
+    s = get_schedule(c, n_orb, true, S);
+    if (s != HFX_OK) return s;
+    *two = pipelined && two_buffers(c, **S);
+    *L = layout_of(c, **S, n_orb, *two);
+    if (*two && c->ws_bytes < L->total) {
+      *two = false;
+      *L = layout_of(c, **S, n_orb, false);
+    }
+    if (c->ws_bytes >= L->total) return HFX_OK;
+  }
+  return fail(HFX_ERR_OOM, "workspace too small: have %zu bytes, need %zu (hfx_workspace_bytes)", c->ws_bytes, need);
 }
 
 // ------------------------------------------------------------------------------------
@@ -1386,12 +1435,11 @@ static hfx_status apply_impl(hfx_ctx* c, const void* orbitals, int32_t n_orb, co
   if (s != HFX_OK) return s;
   if (n_pairs == 0) return apply_empty(c, n_orb, flags, ex_dev, vxphi, st);
   Schedule* S = nullptr;
-  s = get_schedule(c, n_orb, &S);
+  Layout L;
+  bool two = false;
+  s = fit_workspace(c, n_orb, true, &S, &L, &two);
   if (s != HFX_OK) return s;
-  const Layout L = layout_of(c, *S, n_orb, two_buffers(c, *S));
-  if (!c->ws || c->ws_bytes < L.total)
-    return fail(HFX_ERR_OOM, "workspace too small: have %zu bytes, need %zu (hfx_workspace_bytes)", c->ws_bytes, L.total);
-  const CallEnv env{(char*)c->ws, c->side, c->prof_on};
+  const CallEnv env{(char*)c->ws, two ? c->side : nullptr, c->prof_on};
   return apply_with(c, *S, L, env, orbitals, n_orb, pairs, n_pairs, flags, ex_dev, vxphi, st);
 }
 
@@ -1416,6 +1464,15 @@ extern "C" hfx_status hfx_apply_sequential(hfx_ctx* const* ctxs, const hfx_apply
     }
   }
   return HFX_OK;
+}
+
+// the schedule and layout of problem k of a batch: one transform buffer
+static hfx_status fit_problem(hfx_ctx* c, int32_t k, int32_t n_orb, Schedule** S, Layout* L) {
+  bool two;
+  const hfx_status s = fit_workspace(c, n_orb, false, S, L, &two);
+  if (s == HFX_OK) return s;
+  const std::string m = g_last_error;
+  return fail(s, "problem %d: %s", (int)k, m.c_str());
 }
 
 // device tables of the persistent launch: queue header and done counters, tasks, problems
@@ -1466,11 +1523,9 @@ static hfx_status batched_persistent(hfx_ctx* const* ctxs, const hfx_apply_args*
       continue;
     }
     Schedule* S = nullptr;
-    hfx_status s = get_schedule(c, a.n_orb, &S);
+    Layout L;
+    hfx_status s = fit_problem(c, k, a.n_orb, &S, &L);
     if (s != HFX_OK) return s;
-    const Layout L = layout_of(c, *S, a.n_orb, false);
-    if (!c->ws || c->ws_bytes < L.total)
-      return fail(HFX_ERR_OOM, "problem %d: workspace too small: have %zu bytes, need %zu", (int)k, c->ws_bytes, L.total);
     const CallEnv env{(char*)c->ws, nullptr, false};
     const void* orb = nullptr;
     s = stage_call(c, *S, L, env, a.orbitals, a.n_orb, a.pairs, a.n_pairs, a.flags, a.vxphi, st, &orb);
@@ -1615,6 +1670,7 @@ static bool batch_is_small(hfx_ctx* const* ctxs, const hfx_apply_args* args, int
 // (its tables are sized too, so a batch of this size can be captured in either form from then on).
 static hfx_status batched_forked(hfx_ctx* const* ctxs, const hfx_apply_args* args, int32_t n, cudaStream_t st) {
   std::vector<Schedule*> scheds(n, nullptr);
+  std::vector<Layout> layouts(n);
   size_t ntasks = 0, nprobs = 0;
   for (int32_t k = 0; k < n; ++k) {
     hfx_ctx* c = ctxs[k];
@@ -1624,11 +1680,8 @@ static hfx_status batched_forked(hfx_ctx* const* ctxs, const hfx_apply_args* arg
     const size_t planes = std::max(smem_fwd(c), smem_x(c));
     if (planes + 1024 > (size_t)c->max_smem)  // (the limit of the persistent form)
       return fail(HFX_ERR_UNSUPPORTED_GRID, "a batch tile needs %zu bytes of shared memory (limit %d)", planes, c->max_smem);
-    hfx_status s = get_schedule(c, args[k].n_orb, &scheds[k]);
+    hfx_status s = fit_problem(c, k, args[k].n_orb, &scheds[k], &layouts[k]);
     if (s != HFX_OK) return s;
-    const size_t need = layout_of(c, *scheds[k], args[k].n_orb, false).total;
-    if (!c->ws || c->ws_bytes < need)
-      return fail(HFX_ERR_OOM, "problem %d: workspace too small: have %zu bytes, need %zu", (int)k, c->ws_bytes, need);
     const size_t acc = args[k].flags & HFX_ENERGY_ONLY ? 0 : 1;
     ntasks += scheds[k]->nbatches * (2 + acc) + (c->prec == HFX_PREC_FP32 ? acc : 0) + 1;
     ++nprobs;
@@ -1650,7 +1703,7 @@ static hfx_status batched_forked(hfx_ctx* const* ctxs, const hfx_apply_args* arg
     HFX_CUDA_TRY(cudaStreamWaitEvent(c->side, ctxs[0]->ev_fork, 0));
     CallEnv env{(char*)c->ws, nullptr, false};
     env.simt_fwd = true;
-    result = apply_with(c, *scheds[k], layout_of(c, *scheds[k], a.n_orb, false), env, a.orbitals, a.n_orb, a.pairs,
+    result = apply_with(c, *scheds[k], layouts[k], env, a.orbitals, a.n_orb, a.pairs,
                         a.n_pairs, a.flags, a.ex_dev, a.vxphi, c->side);
     // joined also after a failed launch: the caller's stream (or its capture) waits for what was enqueued
     HFX_CUDA_TRY(cudaEventRecord(c->ev_p2, c->side));
@@ -1911,7 +1964,7 @@ extern "C" hfx_status hfx_set_tuning(hfx_ctx* c, int32_t block, size_t batch_byt
     c->gen_phi = old_phi;
     return fail(HFX_ERR_INVALID_ARG, "block %d does not fit this grid's shared-memory tiles", (int)block);
   }
-  c->transform_budget = batch_bytes;
+  c->transform_budget = c->lean_budget = batch_bytes;
   c->pipeline = pipeline != 0;
   // cached schedules depend on the block size and the budget: drop them (device tables freed after
   // the device is idle, since a call in flight may still read them)

@@ -29,7 +29,7 @@ HFX_ORBITALS_F32 = 0x4
 HFX_TEST_STALL = 0x100
 
 # every symbol include/hfx.h and include/hfx_ace.h declare
-EXPORTED = ("hfx_create", "hfx_workspace_bytes", "hfx_set_workspace", "hfx_apply", "hfx_apply_batched",
+EXPORTED = ("hfx_create", "hfx_workspace_bytes", "hfx_workspace_bytes_least", "hfx_set_workspace", "hfx_apply", "hfx_apply_batched",
             "hfx_apply_sequential", "hfx_set_wait_budget", "hfx_apply_noalloc", "hfx_sync_status", "hfx_set_tuning", "hfx_plan_stats", "hfx_profile_enable",
             "hfx_profile_read",
             "hfx_last_error", "hfx_destroy",
@@ -84,6 +84,8 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
     L.hfx_create.restype = ctypes.c_int
     L.hfx_workspace_bytes.argtypes = [vp, i32, i64]
     L.hfx_workspace_bytes.restype = sz
+    L.hfx_workspace_bytes_least.argtypes = [vp, i32, i64]
+    L.hfx_workspace_bytes_least.restype = sz
     L.hfx_set_workspace.argtypes = [vp, vp, sz]
     L.hfx_set_workspace.restype = ctypes.c_int
     L.hfx_apply.argtypes = [vp, vp, i32, vp, i64, u32, vp, vp, vp]
@@ -186,6 +188,10 @@ def hfx_create(lattice, grid: Sequence[int], ecut: float = 0.0, kernel: str = "c
 
 def hfx_workspace_bytes(ctx, n_orb: int, n_pairs: int) -> int:
     return int(load_library().hfx_workspace_bytes(ctx, int(n_orb), int(n_pairs)))
+
+
+def hfx_workspace_bytes_least(ctx, n_orb: int, n_pairs: int) -> int:
+    return int(load_library().hfx_workspace_bytes_least(ctx, int(n_orb), int(n_pairs)))
 
 
 def hfx_set_workspace(ctx, buf: torch.Tensor) -> None:
@@ -360,6 +366,7 @@ class Exchange:
         self.ctx = hfx_create(self.lattice, self.grid, ecut, kernel, alpha, precision)
         self.device = torch.device("cuda", torch.cuda.current_device())
         self._ws: Optional[torch.Tensor] = None
+        self._ws_refused = float("inf")  # the smallest workspace that there was no memory for
 
     @property
     def volume(self) -> float:
@@ -371,10 +378,24 @@ class Exchange:
         return self.grid[0] * self.grid[1] * self.grid[2]
 
     def ensure_workspace(self, n_orb: int, n_pairs: int) -> None:
+        """A workspace of hfx_workspace_bytes or, where the device has no room for one, of
+        hfx_workspace_bytes_least."""
         need = hfx_workspace_bytes(self.ctx, n_orb, n_pairs)
-        if self._ws is None or self._ws.numel() < need:
-            self._ws = torch.empty(max(need, 256), dtype=torch.uint8, device=self.device)
-            hfx_set_workspace(self.ctx, self._ws)
+        if self._ws is not None and self._ws.numel() >= need:
+            return
+        ws = None
+        if need < self._ws_refused:
+            try:
+                ws = torch.empty(max(need, 256), dtype=torch.uint8, device=self.device)
+            except torch.cuda.OutOfMemoryError:
+                self._ws_refused = need
+        if ws is None:
+            least = hfx_workspace_bytes_least(self.ctx, n_orb, n_pairs)
+            if self._ws is not None and self._ws.numel() >= least:
+                return
+            ws = torch.empty(max(least, 256), dtype=torch.uint8, device=self.device)
+        self._ws = ws
+        hfx_set_workspace(self.ctx, self._ws)
 
     def apply(self, phi: torch.Tensor, pairs: torch.Tensor, energy_only: bool = False, accumulate: bool = False,
               ex: Optional[torch.Tensor] = None, vxphi: Optional[torch.Tensor] = None,
