@@ -121,7 +121,7 @@ hfx_status hfx_create(const hfx_box* box, const int32_t grid[3], double ecut, hf
 size_t hfx_workspace_bytes(const hfx_ctx* c, int32_t n_orb, int64_t n_pairs);
 
 /* hfx_workspace_bytes_least -- the least workspace that hfx_apply accepts, for a device without room for
- * hfx_workspace_bytes: batches of at most 1 GiB of transforms (of batch_bytes after hfx_set_tuning), each with
+ * hfx_workspace_bytes: batches of at most 1 GiB of transforms (and of batch_bytes, hfx_set_tuning), each with
  * launches of its own (the first such call for an n_orb uploads its schedule table, as the first call of all
  * does).  A call takes what the workspace holds; results do not depend on it beyond rounding
  * order, times do: 256 orbitals on 96^3 take 138 ms in 5.9 GB and 144 to 149 in 3.9 GB, 64 on 64^3 2.4 ms

@@ -179,9 +179,6 @@ struct hfx_ctx {
   // orbitals on 96^3 took 150.3, 145.2, 137.6 and 135.5 ms with 0.5, 1, 2 and 4 GiB, 64 on 128^3 29.0, 27.4,
   // 26.3 and 26.3; rounds that fit 1 GiB (72^3) do not change
   size_t transform_budget = size_t(2) << 30;
-  // the same for a workspace that does not hold such batches (hfx_workspace_bytes_least); what the caller sets
-  // is for both
-  size_t lean_budget = size_t(1) << 30;
   int blocks_fwd = 1, blocks_x = 1;
   int gen_grp = 1, gen_phi = 0;  // generic accumulate pass: couples per group, orbital tiles on chip
   // second stream and events: the forward and x passes of batch b+1 run beside the accumulate
@@ -625,7 +622,7 @@ extern "C" hfx_status hfx_create(const hfx_box* box, const int32_t grid[3], doub
   c->alpha = alpha;
   c->prec = prec;
   if (const char* s = std::getenv("HFX_BLOCK")) c->bsize = std::max(1, std::min(32, atoi(s)));
-  if (const char* s = std::getenv("HFX_BATCH_MB")) c->transform_budget = c->lean_budget = (size_t)std::max(1, atoi(s)) << 20;
+  if (const char* s = std::getenv("HFX_BATCH_MB")) c->transform_budget = (size_t)std::max(1, atoi(s)) << 20;
   if (const char* s = std::getenv("HFX_PIPELINE")) c->pipeline = atoi(s) != 0;
   if (const char* s = std::getenv("HFX_NO_TC")) c->ace_tc = atoi(s) == 0;
   if (const char* s = std::getenv("HFX_DENSE_TMA")) c->dense_tma = atoi(s) != 0;
@@ -757,10 +754,12 @@ static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 // 666; together lost at 48^3 with 24 (201 / 221) and 32^3 with 64 (371 / 409), whose batches are 44 and 33 MB.
 constexpr size_t kGroupMin = size_t(64) << 20, kGroupMax = size_t(1) << 30;
 
-// lean: batches of at most lean_budget, a launch each, for a workspace that does not hold the others
+// lean: batches of at most kLeanBudget with launches of their own, for a workspace that does not hold the
+// others (hfx_workspace_bytes_least)
+constexpr size_t kLeanBudget = size_t(1) << 30;
 static Schedule make_host_schedule(const hfx_ctx* c, int n_orb, bool lean = false) {
   Schedule S;
-  const size_t per = (size_t)c->N * cplx_size(c), budget = lean ? c->lean_budget : c->transform_budget;
+  const size_t per = (size_t)c->N * cplx_size(c), budget = lean ? std::min(kLeanBudget, c->transform_budget) : c->transform_budget;
   build_schedule(S, n_orb, c->bsize, budget, per, dense_available(c), diag_available(c), ragged_rows(c));
   S.dead_words = ragged_dense(c);
   build_groups(S, !lean && c->ct && S.max_batch_couples * per >= kGroupMin ? (long long)(std::min(kGroupMax, budget) / per) : 0);
@@ -1964,7 +1963,7 @@ extern "C" hfx_status hfx_set_tuning(hfx_ctx* c, int32_t block, size_t batch_byt
     c->gen_phi = old_phi;
     return fail(HFX_ERR_INVALID_ARG, "block %d does not fit this grid's shared-memory tiles", (int)block);
   }
-  c->transform_budget = c->lean_budget = batch_bytes;
+  c->transform_budget = batch_bytes;
   c->pipeline = pipeline != 0;
   // cached schedules depend on the block size and the budget: drop them (device tables freed after
   // the device is idle, since a call in flight may still read them)

@@ -38,6 +38,7 @@ EXPORTED = ("hfx_create", "hfx_workspace_bytes", "hfx_workspace_bytes_least", "h
             "hfx_sinr_update_n", "hfx_sinr_update_v", "hfx_sinr_update_x", "hfx_fma_peak",
             "hfx_debug_check_guards", "hfx_test_fail_allocation", "hfx_test_live_allocations")
 HFX_NOALLOC_SCRATCH_BYTES = 32 << 20
+DEFAULT_BATCH_BYTES = 2 << 30  # the library's own default (hfx_set_tuning)
 PASS_NAMES = ("stage", "fwd_yz", "x_coulomb", "y_acc_dense", "energy", "y_acc_generic")
 ACE_KERNEL_NAMES = ("ace_gram", "ace_lmul", "ace_small")
 
@@ -246,7 +247,7 @@ def hfx_sync_status(ctx, stream: Optional[torch.cuda.Stream] = None) -> None:
     _check(load_library().hfx_sync_status(ctx, _stream_handle(stream)))
 
 
-def hfx_set_tuning(ctx, block: int = 8, batch_bytes: int = 1 << 30, pipeline: bool = True) -> None:
+def hfx_set_tuning(ctx, block: int = 8, batch_bytes: int = DEFAULT_BATCH_BYTES, pipeline: bool = True) -> None:
     _check(load_library().hfx_set_tuning(ctx, int(block), int(batch_bytes), 1 if pipeline else 0))
 
 
@@ -495,7 +496,7 @@ class Exchange:
         hfx_screen_pairs(self.ctx, phi, cut, s, pairs, count, self._ace_workspace(n, 0), stream)
         return pairs[: int(count.item())], s
 
-    def set_tuning(self, block: int = 8, batch_bytes: int = 1 << 30, pipeline: bool = True) -> None:
+    def set_tuning(self, block: int = 8, batch_bytes: int = DEFAULT_BATCH_BYTES, pipeline: bool = True) -> None:
         hfx_set_tuning(self.ctx, block, batch_bytes, pipeline)
         self.tuning = {"block": int(block), "batch_bytes": int(batch_bytes), "pipeline": bool(pipeline)}
 
