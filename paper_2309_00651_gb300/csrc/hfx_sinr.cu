@@ -31,7 +31,8 @@ namespace {
 // freedom of 128 H2O) is spread over as many SMs as it has warps, and only a large one uses full blocks.
 // With 256 threads and the chain in local memory an update A of 1152 degrees of freedom (chain 4, three
 // factors) took 31 us, of 20000 31; now 15 and 23.  Large systems are bound by the FP64 pipe as before
-// (10^6: 697 us).
+// (10^6: 697 us).  These calls have no context to ask for the SM count; another one only spreads the warps
+// differently.
 constexpr int kSms = 152;
 constexpr int kMaxThreads = 256;
 int block_threads(long long n) {
@@ -69,16 +70,16 @@ __global__ void __launch_bounds__(kMaxThreads) k_update_n(SinrArgs a, long long 
       // e_j = exp(-v2_j Delta/2) serves both the rescaling of v1 and, squared, the denominator of H
       double e[ML];
       double den = M * vel * vel;
-    #pragma unroll
-  for (int j = 0; j < L; ++j) {
+#pragma unroll
+      for (int j = 0; j < L; ++j) {
         x2[j] += c * fma(a.Q1 * x1[j], x1[j], -a.kT);
         e[j] = exp(hd * x2[j]);
         den += cq * (x1[j] * x1[j]) * (e[j] * e[j]);
       }
       const double H = sqrt_lam * rsqrt(den);
       vel *= H;
-    #pragma unroll
-  for (int j = 0; j < L; ++j) {
+#pragma unroll
+      for (int j = 0; j < L; ++j) {
         x1[j] *= H * e[j];
         x2[j] += c * fma(a.Q1 * x1[j], x1[j], -a.kT);
       }
