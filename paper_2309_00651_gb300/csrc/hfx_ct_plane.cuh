@@ -37,9 +37,20 @@ namespace ct {
 template <int N> struct PlaneGeo {
   static_assert(N % 4 == 0, "plane passes need an edge that is a multiple of 4");
   static constexpr int R = N / 4;                                   // large radix of z and x
-  // forward rows without gaps, where that lets another plane fit an SM
-  static constexpr bool kDense = R == 24;
-  static constexpr int E = kDense ? R : (R + 3) / 8 * 8 + 4;        // >= R, 4 mod 8
+  static constexpr StagePlan Y = stage_plan(N);
+  static_assert(Y.ns == 2, "two y stages");
+  static constexpr int RY0 = Y.r[0], RY1 = Y.r[1];
+  static constexpr int TW = 4 * (R + R % 2);                        // z and x twiddles, then y's
+  static constexpr int TWY = RY1 * RY0;
+  // dynamic shared memory of the forward pass for a row stride, and how many such planes fit an SM (228 KB,
+  // of which each block takes 1 KB more than it asks for)
+  static constexpr int fwd_bytes(int stride) { return (N * stride + TW + TWY) * 8; }
+  static constexpr int fwd_planes(int stride) { return 228 * 1024 / (fwd_bytes(stride) + 1024); }
+  static constexpr int kPadE = (R + 3) / 8 * 8 + 4;                 // >= R, 4 mod 8
+  // forward rows without gaps, where the digits then lie 8 mod 16 apart (eight rows x two e cover the banks)
+  // and a third plane fits an SM that holds two (96 so far); with more planes than that latency is hidden anyway
+  static constexpr bool kDense = R % 16 == 8 && fwd_planes(4 * kPadE + 3) <= 2 && fwd_planes(4 * R + 1) > fwd_planes(4 * kPadE + 3);
+  static constexpr int E = kDense ? R : kPadE;
   static constexpr int SF = 4 * E + (kDense ? 1 : 3);               // forward row stride
   // row and z digit of task `id` of the z stage
   static __device__ __forceinline__ void z_task(int id, int& y, int& e) {
@@ -52,17 +63,12 @@ template <int N> struct PlaneGeo {
     }
   }
   static constexpr int SX = N + 2;                                  // x-pass row stride
-  static constexpr StagePlan Y = stage_plan(N);
-  static_assert(Y.ns == 2, "two y stages");
-  static constexpr int RY0 = Y.r[0], RY1 = Y.r[1];
-  static constexpr int TW = 4 * (R + R % 2);                        // z and x twiddles, then y's
-  static constexpr int TWY = RY1 * RY0;
   static_assert(E >= R && (kDense || E % 8 == 4), "bank-spreading stride of the z digits");
   // place of output k of the large radix among its R: as two radices the runtime-geometry kernels know
   // (plane_radices) would leave it, so that the tables and the pencil and batch kernels share the order
   static constexpr PlaneRadices P = plane_radices(R);
   static __host__ __device__ constexpr int place(int k) { return (k % P.a) * P.b + k / P.a; }
-  static constexpr int smem_fwd = (N * SF + TW + TWY) * 8;
+  static constexpr int smem_fwd = fwd_bytes(SF);
   static constexpr int smem_x = (N * SX + 2 + TW) * 8;
 };
 
