@@ -379,9 +379,15 @@ static bool ragged_dense(const hfx_ctx* c) {
 }
 
 // whether the dense pass in use takes the ragged last block's pairs: the TMA form and the runtime-geometry
-// form do (27 orbitals on 54x60x72: call 1.33 -> 1.30 ms), the compile-time form with per-thread copies does not
-static bool ragged_rows(const hfx_ctx* c) {
-  return ragged_dense(c) || (dense_available(c) && !(c->ct && c->bsize == 8));
+// form do (27 orbitals on 54x60x72: call 1.33 -> 1.30 ms), the compile-time form with per-thread copies does not.
+// With three blocks a round is one such pair and a diagonal one, which the generic pass takes in one launch, so
+// the runtime-geometry form pays from about 20^3 points on: generic / dense and generic, us a call of 20
+// orbitals, FP64: 8^3 145 / 188, 12^3 238 / 260, 16^3 380 / 380, 20^3 506 / 472, 30^3 964 / 863; FP32 98 / 106,
+// 107 / 110, 130 / 131, 164 / 164, 220 / 199.  With two or four blocks it gains 10 to 25% from 8^3 on.
+static bool ragged_rows(const hfx_ctx* c, int n_orb) {
+  if (ragged_dense(c)) return true;
+  const int nb = (n_orb + c->bsize - 1) / c->bsize;
+  return dense_available(c) && !(c->ct && c->bsize == 8) && !(nb == 3 && c->N < 20 * 20 * 20);
 }
 
 // Every device allocation the library makes for itself (context tables, schedules, batch tables)
@@ -760,7 +766,7 @@ constexpr size_t kLeanBudget = size_t(1) << 30;
 static Schedule make_host_schedule(const hfx_ctx* c, int n_orb, bool lean = false) {
   Schedule S;
   const size_t per = (size_t)c->N * cplx_size(c), budget = lean ? std::min(kLeanBudget, c->transform_budget) : c->transform_budget;
-  build_schedule(S, n_orb, c->bsize, budget, per, dense_available(c), diag_available(c), ragged_rows(c));
+  build_schedule(S, n_orb, c->bsize, budget, per, dense_available(c), diag_available(c), ragged_rows(c, n_orb));
   S.dead_words = ragged_dense(c);
   build_groups(S, !lean && c->ct && S.max_batch_couples * per >= kGroupMin ? (long long)(std::min(kGroupMax, budget) / per) : 0);
   return S;
@@ -1914,7 +1920,7 @@ extern "C" hfx_status hfx_apply_noalloc(hfx_ctx* c, const void* orbitals, int32_
     const size_t room = fixed < kNoallocScratchBytes ? kNoallocScratchBytes - fixed : 0;
     if (room >= (size_t)cap_max * couple_bytes + 256) {
       build_schedule(S, n_orb, c->bsize, room - 256, couple_bytes, dense_available(c), diag_available(c),
-                     ragged_rows(c));
+                     ragged_rows(c, n_orb));
       S.dead_words = ragged_dense(c);
       build_groups(S, 0);
       L = layout_of(c, S, n_orb, false);
