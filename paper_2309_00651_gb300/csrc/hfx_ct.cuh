@@ -201,10 +201,10 @@ __device__ __forceinline__ void two_sum(float& s, float& e, float a, float ea) {
 // A plane's energy: each thread adds its FP32 partials, one per butterfly, with their rounding errors carried
 // along, then a tree per warp into red and one over the warps do the same (about 48 bits).  So the only FP32
 // roundings are those inside a butterfly, as in the runtime-geometry pass, whose other sums are FP64.  Those
-// would take the narrow FP64 pipe here; plain FP32 sums were up to 2e-8 off (64^3, F = 1 everywhere:
-// 9e-9 rms over eight cells, now 1e-9).  Against those the x pass takes up to 1% more, 1.8% at 80^3
-// (64 orbitals, us a call, plain / this: 64^3 857 / 866, 72^3 1373 / 1387, 80^3 1882 / 1914, 96^3 3904 / 3950,
-// 128^3, 32 orbitals, 2746 / 2772).
+// would take the narrow FP64 pipe here; plain FP32 sums were up to 2e-8 off (64^3, F = 1 everywhere: 9e-9 rms
+// over eight cells, now 1e-9).  Against plain sums the x pass takes up to 3% more, us for 256 couples: 24.4 / 25.2
+// (32^3), 85.6 / 87.2 (48^3), 209.3 / 211.7 (64^3), 337.7 / 342.4 (72^3), 469 / 472 (80^3), 877 / 892 (96^3), 2356 /
+// 2366 (128^3).
 struct PlaneSum {
   float s = 0.f, e = 0.f;
   __device__ __forceinline__ void add(float a) { two_sum(s, e, a, 0.f); }

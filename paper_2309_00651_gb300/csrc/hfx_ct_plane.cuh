@@ -13,15 +13,16 @@
 // Measured against the one-stage-at-a-time form, us per launch of 256 couples: forward / x pass 45 / 45
 // -> 28 / 27 (32^3), 108 / 127 -> 90 / 96 (48^3), 231 / 239 -> 194 / 221 (64^3), 338 / 409 -> 292 / 346
 // (72^3), 436 / 531 -> 415 / 472 (80^3), 778 / 1012 -> 676 / 892 (96^3), 2262 / 2872 -> 2075 / 2368
-// (128^3).  At 72^3 the x pass moves 4.4 TB/s of DRAM; with its loads and stores taken out it runs in
-// 252 us, with its shared-memory stages taken out in 254, so what is left is how far the two overlap.
+// (128^3), before the energy sums of PlaneSum.  At 72^3 the x pass moves 4.4 TB/s of DRAM; with its loads and
+// stores taken out it runs in 252 us, with its shared-memory stages taken out in 254, so what is left is how far
+// the two overlap.
 //
 // Layouts, chosen so that the half-warps of every stage touch 16 different 8-byte banks:
 //   forward: z = 4 D + e of row y sits at y S + e E + D (E = 4 or 12 mod 16, S = 3 mod 16): four rows x
 //            four e of the z stage, runs of D in the last stage, and runs of (D, e) in the y stage.
-//            At 96^3 rows go without gaps (E = 24 = 8, S = 97 = 1 mod 16, eight rows x two e in the z stage,
-//            runs of places in the y stage), so that three planes fit an SM instead of two: 721 -> 676 us (at
-//            72^3 a fifth plane by rows without gaps lost, 288 -> 302 us);
+//            At 96^3 rows go without gaps (kDense; E = 24 = 8, S = 97 = 1 mod 16, eight rows x two e in the z
+//            stage, runs of places in the y stage), so that three planes fit an SM instead of two: 721 -> 676 us
+//            (at 72^3 a fifth plane by rows without gaps lost, 288 -> 302 us);
 //   x pass:  (x, z) sits at x S + z + 2 ((x / 8) mod 2), S = N + 2 (2 or 10 mod 16): eight rows x two z
 //            in the z stage, runs of z in the x stages, and in the tile stage 16-byte accesses of which
 //            eight consecutive lanes (two x, four z tiles) cover all banks.
@@ -49,7 +50,8 @@ template <int N> struct PlaneGeo {
   static constexpr int kPadE = (R + 3) / 8 * 8 + 4;                 // >= R, 4 mod 8
   // forward rows without gaps, where the digits then lie 8 mod 16 apart (eight rows x two e cover the banks)
   // and a third plane fits an SM that holds two (96 so far); with more planes than that latency is hidden anyway
-  static constexpr bool kDense = R % 16 == 8 && fwd_planes(4 * kPadE + 3) <= 2 && fwd_planes(4 * R + 1) > fwd_planes(4 * kPadE + 3);
+  static constexpr bool kDense =
+      R % 16 == 8 && fwd_planes(4 * kPadE + 3) <= 2 && fwd_planes(4 * R + 1) > fwd_planes(4 * kPadE + 3);
   static constexpr int E = kDense ? R : kPadE;
   static constexpr int SF = 4 * E + (kDense ? 1 : 3);               // forward row stride
   // row and z digit of task `id` of the z stage
@@ -128,7 +130,9 @@ __device__ __forceinline__ void product_to_smem(const float* __restrict__ orb, l
   using G = PlaneGeo<N>;
   constexpr int NV = N * G::R;
   const bool hasa = cp.x >= 0, hasb = cp.z >= 0;
-  const bool same = cp.x == cp.z;  // full couples of an off-diagonal block pair hold (i, j) and (i, j + 1)
+  // full couples of an off-diagonal block pair hold (i, j) and (i, j + 1): three planes are read.  Those of a
+  // ragged block pair hold (i, j) and (i + 1, j) and read four.
+  const bool same = cp.x == cp.z;
   const long long off = (long long)x * (N * N);
   const float4* a1 = reinterpret_cast<const float4*>(orb + (long long)(hasa ? cp.x : 0) * Ntot + off);
   const float4* a2 = reinterpret_cast<const float4*>(orb + (long long)(hasa ? cp.y : 0) * Ntot + off);
