@@ -268,7 +268,7 @@ hfx_status hfx_sync_status(hfx_ctx* c, void* cuda_stream);
 hfx_status hfx_set_tuning(hfx_ctx* c, int32_t block, size_t batch_bytes, int32_t pipeline);
 
 /* hfx_plan_stats -- what hfx_apply(c, ..., n_orb, ..., n_pairs, flags, ...) will launch, from the
- * host schedule alone (no device work):
+ * host schedule alone (no device work; a workspace of hfx_workspace_bytes):
  *   out[0] = kernel launches per call, out[1] = batches, out[2] = orbital block size,
  *   out[3] = largest number of packed pair couples (two pairs per complex 3D transform) held
  *   by one batch, out[4] = couples of the whole call when every block pair is full (the
