@@ -137,7 +137,9 @@ size_t hfx_workspace_bytes_least(const hfx_ctx* c, int32_t n_orb, int64_t n_pair
 hfx_status hfx_set_workspace(hfx_ctx* c, void* dev_ptr, size_t bytes);
 
 /* hfx_apply -- one exact-exchange evaluation (Eqs. vx, vij, HFX).
- *   orbitals : device, [n_orb][n1][n2][n3], FP64 (FP32 with HFX_ORBITALS_F32); read only.
+ *   orbitals : device, [n_orb][n1][n2][n3], FP64 (FP32 with HFX_ORBITALS_F32); read only.  Every
+ *              orbital holds finite values, also one that no pair lists: an infinity or a NaN can
+ *              reach V_x phi of other orbitals, whether a pair joins the two or not.
  *   n_orb    : number of occupied orbitals (> 0).
  *   pairs    : device int32 [n_pairs][2], entries 0 <= i <= j < n_orb, any order (Sec. 2.1
  *              screening: any subset of pairs may be listed).  Invalid entries are skipped
